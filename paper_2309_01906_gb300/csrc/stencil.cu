@@ -15,6 +15,9 @@
 // the array forced to 0), and stores only its tile.  Every point of every step
 // is one FP32 FMA chain over the window in row-major order from 0, so a run of
 // T steps equals T runs of one step bit for bit.
+//
+// Maps that leave tiles and sections automatic run the register-streamed
+// kernels of stencil_stream.cuh instead (the same chains, the same bits).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -27,6 +30,7 @@
 #include <vector>
 
 #include "hp_internal.h"
+#include "stencil_stream.h"
 
 namespace hp {
 
@@ -48,7 +52,14 @@ struct StencilPlan {
   int64_t tiles_y = 0, tiles_x = 0;
   std::vector<int32_t> order;    // tiles (ty, tx) pairs, section after section
   float c[(2 * kStencilMaxR + 1) * (2 * kStencilMaxR + 1)] = {};
+  bool stream = false;           // tiles and sections automatic, and a streamed kernel exists
   size_t smem() const { return static_cast<size_t>(nbuf) * buf_floats * sizeof(float); }
+  // Does a run take the streamed kernel?  Steps kept in registers beat steps
+  // kept in shared memory everywhere (16384^2, radius 1, 4 steps: 443 us
+  // against 1026; radius 4, one step: 719 against 1410) but one aligned step of
+  // radius 1, which both run at the memory's rate and the tiles' large tensor
+  // copies read a little faster (334 us against 357).
+  bool streamed(bool vec) const { return stream && !(r == 1 && T == 1 && vec); }
 };
 
 namespace {
@@ -124,6 +135,8 @@ hp_status plan_stencil(int64_t ny, int64_t nx, int radius, const float* coeffs, 
           p.order.push_back(static_cast<int32_t>(ty));
           p.order.push_back(static_cast<int32_t>(tx));
         }
+  p.stream = stream_has(radius, steps) &&
+             (!map || (!map->tile_y && !map->tile_x && !map->section_y && !map->section_x));
   *out = std::move(p);
   return HP_OK;
 }
@@ -133,7 +146,9 @@ std::string describe_stencil(const StencilPlan& p) {
   s << "{\"kind\":\"stencil\",\"ny\":" << p.ny << ",\"nx\":" << p.nx << ",\"radius\":" << p.r << ",\"steps\":" << p.T
     << ",\"tile\":[" << p.TY << "," << p.TX << "],\"ghost\":[" << p.h << "," << p.hx << "],\"box\":[" << p.boxH << ","
     << p.boxW << "],\"buffers\":" << p.nbuf << ",\"smem\":" << p.smem() << ",\"tiles\":" << p.order.size() / 2
-    << ",\"section\":[" << p.SY << "," << p.SX << "]";
+    << ",\"section\":[" << p.SY << "," << p.SX << "],\"kernel\":\""
+    << (p.streamed(p.nx % 4 == 0) ? "stencil_stream" : "stencil_tile") << "\"";
+  if (p.stream) s << ",\"warp_columns\":" << stream_columns(p.r, p.T);
   const int64_t secs_y = (p.ny + p.SY - 1) / std::max<int64_t>(p.SY, 1), secs_x = (p.nx + p.SX - 1) / std::max<int64_t>(p.SX, 1);
   if (p.ny > 0 && p.nx > 0 && secs_y * secs_x <= 64) {
     // the GRID level's map sections: `to` = section + ghost border (clipped), `from` = section (clipped)
@@ -370,6 +385,7 @@ struct hp_stencil {
   int sms = 0;
   int32_t* d_order = nullptr;
   int32_t* err = nullptr;
+  uint32_t strip[2] = {0, 0};    // streamed kernels: rows per strip (scalar rows, 16-byte rows)
   std::mutex mu;                 // guards the cached tensor map
   CUtensorMap tmap;
   const float* tmap_ptr = nullptr;
@@ -453,6 +469,12 @@ hp_status stencil_ensure_device(hp_stencil* s) {
     return stencil_cuda_fail(e, "upload tile order");
   if ((e = cudaMalloc(&s->err, sizeof(int32_t))) != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (error word)");
   if ((e = cudaMemset(s->err, 0, sizeof(int32_t))) != cudaSuccess) return stencil_cuda_fail(e, "cudaMemset");
+  const StencilPlan& p = s->plan;
+  for (int vec = 0; p.stream && vec < 2; ++vec) {
+    const int ctas = stream_occupancy(p.r, p.T, vec != 0, &e);
+    if (e != cudaSuccess) return stencil_cuda_fail(e, "occupancy query");
+    s->strip[vec] = stream_strip_rows(p.ny, p.nx, p.r, p.T, std::max(ctas, 1), s->sms);
+  }
   s->device = dev;
   return HP_OK;
 }
@@ -488,6 +510,22 @@ extern "C" hp_status hp_stencil_run(hp_stencil* s, const float* in_dev, float* o
   if (a < b + bytes && b < a + bytes) return fail(HP_EINVAL, "in and out overlap (the stencil runs out of place)");
   hp_status st = stencil_ensure_device(s);
   if (st != HP_OK) return st;
+  cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  cudaError_t e;
+  const bool vec = p.nx % 4 == 0 && reinterpret_cast<uintptr_t>(in_dev) % 16 == 0 &&
+                   reinterpret_cast<uintptr_t>(out_dev) % 16 == 0;
+  if (p.streamed(vec)) {
+    StreamArgs a;
+    a.in = in_dev;
+    a.out = out_dev;
+    a.ny = static_cast<uint32_t>(p.ny);
+    a.nx = static_cast<uint32_t>(p.nx);
+    a.S = s->strip[vec];
+    std::memcpy(a.c, p.c, sizeof(a.c));
+    e = stream_launch(p.r, p.T, vec, a, cs);
+    if (e != cudaSuccess) return stencil_cuda_fail(e, "stencil launch");
+    return HP_OK;
+  }
   StencilArgs args;
   args.in = in_dev;
   args.out = out_dev;
@@ -517,8 +555,6 @@ extern "C" hp_status hp_stencil_run(hp_stencil* s, const float* in_dev, float* o
     if (args.use_tma) tmap = s->tmap;
     else std::memset(&tmap, 0, sizeof(tmap));
   }
-  cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  cudaError_t e;
   switch (p.r) {
     case 0: e = stencil_launch<0>(tmap, args, p.smem(), s->sms, cs); break;
     case 1: e = stencil_launch<1>(tmap, args, p.smem(), s->sms, cs); break;
