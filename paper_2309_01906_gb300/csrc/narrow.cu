@@ -9,7 +9,9 @@
 // __vmins2) whose sub-lanes are folded once at the end.  Warps combine with
 // the warp-reduce instructions (__reduce_add/max/min_sync), CTAs in shared
 // memory, grid parts after a ticket.  Integer results do not depend on the
-// order, so threads take 16-byte pieces cyclically (coalesced).
+// order, so threads take 16-byte pieces cyclically (coalesced), rows that start
+// or end off a 16-byte boundary give their ends to single-element loads, and
+// short rows share a warp (narrow_rows_kernel).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -22,6 +24,14 @@
 namespace hp {
 
 constexpr int kNarThreads = 256;
+
+// Teams of up to 256 threads are compiled for 8 resident CTAs per SM (32
+// registers): a streaming fold needs the bytes in flight of 2048 threads to
+// keep HBM busy.  Larger CTA teams (sub_width up to 32 warps) take a 1024-thread
+// variant.
+constexpr int kNarMinBlocks = 8;
+constexpr int kNarDotBlocks = 6;   // CTA teams of the dot product: 40 registers (16384 x 65536: 152 us, with 8 CTAs 164)
+
 
 namespace {
 int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -100,7 +110,8 @@ hp_status plan_narrow(int depth, const int64_t* extents, const hp_level_map* map
       if (tile > 0) {
         part = tile * inner;
       } else {
-        const int64_t want = std::max<int64_t>(1, ceil_div64(8 * 152, std::max<int64_t>(O, 1)));
+        // one wave of the CTAs that fit on an SM
+        const int64_t want = std::max<int64_t>(1, (body == HP_BODY_DOT_BCAST ? kNarDotBlocks : kNarMinBlocks) * 152 / std::max<int64_t>(O, 1));
         part = std::max<int64_t>(65536, ceil_div64(R, want));
         const int64_t step = (R % piece == 0) ? inner * piece / gcd64(inner, piece) : inner;   // whole pieces
         part = ceil_div64(part, step) * step;
@@ -151,37 +162,60 @@ struct NarArgs {
   int32_t W;
 };
 
+// the larger (OP 1) or smaller (OP 2) of each signed 16-bit half: one instruction from sm_90 on
+template <int OP>
+__device__ __forceinline__ uint32_t minmax16(uint32_t a, uint32_t b) {
+  uint32_t r;
+  if constexpr (OP == 1) asm("max.s16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  else asm("min.s16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// A thread's running value.  Sums: an int32.  Maxima and minima: packed 16-bit
+// lanes.  A 16-bit comparison is decided by the high byte first, so the high
+// byte of the larger of two 16-bit values is the larger of their high bytes:
+// int8 lanes 1 and 3 of a word fold as they stand, lanes 0 and 2 after a shift by
+// 8 (3 instructions per word; __vmaxs4 is emulated on this GPU: 65536 x 4099
+// int8, 40 us against 47).
 // E: int8_t or int16_t; OP: 0 sum, 1 max, 2 min
 template <class E, int OP>
 struct NarrowOp {
   static constexpr bool kI8 = sizeof(E) == 1;
-  // packed identity of a running max / min register, and the scalar identity
-  static constexpr uint32_t packed_ident() {
-    return OP == 1 ? (kI8 ? 0x80808080u : 0x80008000u) : (kI8 ? 0x7f7f7f7fu : 0x7fff7fffu);
-  }
   static constexpr int32_t ident() { return OP == 0 ? 0 : (OP == 1 ? (kI8 ? -128 : -32768) : (kI8 ? 127 : 32767)); }
+  // the identity in every sub-lane of a word of input
+  static constexpr uint32_t packed_ident() {
+    return OP == 0 ? 0u
+                   : OP == 1 ? (kI8 ? 0x80808080u : 0x80008000u) : (kI8 ? 0x7f7f7f7fu : 0x7fff7fffu);
+  }
+  struct Run {
+    int32_t sum = 0;
+    uint32_t hi = OP == 1 ? 0x80008000u : 0x7fff7fffu, lo = hi;   // lo: int8 lanes 0 and 2
+  };
   // one 32-bit register of the input: 4 (2) sub-lanes
-  __device__ static __forceinline__ void fold_word(uint32_t x, uint32_t wv, int32_t& acc, uint32_t& pk, bool dot) {
+  __device__ static __forceinline__ void fold_word(uint32_t x, uint32_t wv, Run& r, bool dot) {
     if constexpr (OP == 0) {
-      if constexpr (kI8) acc = __dp4a(static_cast<int>(x), dot ? static_cast<int>(wv) : 0x01010101, acc);
-      else acc = __dp2a_lo(static_cast<int>(x), 0x0101, acc);
-    } else if constexpr (kI8) {
-      pk = OP == 1 ? __vmaxs4(pk, x) : __vmins4(pk, x);
-    } else if constexpr (OP == 1) {   // packed 16-bit max / min are native instructions from sm_90 on
-      asm("max.s16x2 %0, %1, %2;" : "=r"(pk) : "r"(pk), "r"(x));
+      if constexpr (kI8) r.sum = __dp4a(static_cast<int>(x), dot ? static_cast<int>(wv) : 0x01010101, r.sum);
+      else r.sum = __dp2a_lo(static_cast<int>(x), 0x0101, r.sum);
     } else {
-      asm("min.s16x2 %0, %1, %2;" : "=r"(pk) : "r"(pk), "r"(x));
+      r.hi = minmax16<OP>(r.hi, x);
+      if constexpr (kI8) r.lo = minmax16<OP>(r.lo, x << 8);
     }
   }
-  __device__ static __forceinline__ int32_t unpack(uint32_t pk) {   // fold the sub-lanes of a packed register
-    int32_t r = ident();
-    const int n = kI8 ? 4 : 2;
-    for (int i = 0; i < n; ++i) {
-      const int32_t v = kI8 ? static_cast<int32_t>(static_cast<int8_t>(pk >> (8 * i)))
-                            : static_cast<int32_t>(static_cast<int16_t>(pk >> (16 * i)));
-      r = OP == 1 ? max(r, v) : min(r, v);
+  __device__ static __forceinline__ void fold_piece(const uint4& q, const uint4& w, Run& r, bool dot) {
+    fold_word(q.x, w.x, r, dot);
+    fold_word(q.y, w.y, r, dot);
+    fold_word(q.z, w.z, r, dot);
+    fold_word(q.w, w.w, r, dot);
+  }
+  __device__ static __forceinline__ int32_t value(const Run& r) {
+    if constexpr (OP == 0) {
+      return r.sum;
+    } else {
+      const uint32_t p = kI8 ? minmax16<OP>(r.hi, r.lo) : r.hi;
+      const int32_t a = static_cast<int32_t>(p) >> (kI8 ? 24 : 16);
+      const int32_t b = static_cast<int32_t>(p << 16) >> (kI8 ? 24 : 16);
+      return combine(a, b);
     }
-    return r;
   }
   __device__ static __forceinline__ int32_t combine(int32_t a, int32_t b) {
     if constexpr (OP == 0) return static_cast<int32_t>(static_cast<uint32_t>(a) + static_cast<uint32_t>(b));
@@ -195,80 +229,119 @@ struct NarrowOp {
   }
 };
 
-// this thread's share of elements [lo, hi) of one output (base = the output's first element)
-template <class E, int OP, bool DOT, bool VEC>
+// bytes s .. s + 15 of the 32 bytes (x, y)
+__device__ __forceinline__ uint4 shift_bytes(uint4 x, uint4 y, uint32_t s) {
+  uint32_t v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+  if (s & 8u) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) v[i] = v[i + 2];
+  }
+  if (s & 4u) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) v[i] = v[i + 1];
+  }
+  const uint32_t b = 8u * (s & 3u);
+  return make_uint4(__funnelshift_r(v[0], v[1], b), __funnelshift_r(v[1], v[2], b), __funnelshift_r(v[2], v[3], b),
+                    __funnelshift_r(v[3], v[4], b));
+}
+
+// This thread's share of elements [lo, hi) of one output (a = the output's
+// first element): whole 16-byte pieces cyclically over the T threads of the
+// team.  RAGGED: the elements before the first and after the last 16-byte
+// boundary go to single loads, one per thread, and a broadcast operand that
+// starts off the pieces' boundary is read as two aligned pieces and shifted
+// (pieces whose two would reach outside w join the single loads).  Rows of
+// 65541 int8, 268 MB: 466 us as single loads, 39 so (HBM's rate); the dot
+// product 465 and 47.
+template <class E, int OP, bool DOT, bool RAGGED>
 __device__ __forceinline__ int32_t fold_range(const E* __restrict__ a, const E* __restrict__ w, int64_t lo, int64_t hi,
-                                              int64_t t, int64_t T) {
+                                              int64_t R, int64_t t, int64_t T) {
   using Op = NarrowOp<E, OP>;
-  int32_t acc = OP == 0 ? 0 : Op::ident();
-  uint32_t pk = Op::packed_ident();
-  if constexpr (VEC) {
-    constexpr int64_t kP = 16 / sizeof(E);   // elements per 128-bit piece
-    const int64_t first = lo / kP + t, pe = hi / kP;
-    const uint4* ap = reinterpret_cast<const uint4*>(a) + first;
-    const uint4* wq = reinterpret_cast<const uint4*>(w) + first;
-    int64_t n = first < pe ? (pe - first + T - 1) / T : 0;   // pieces of this thread
+  constexpr int64_t kP = 16 / sizeof(E);   // elements per 128-bit piece
+  typename Op::Run run;
+  int32_t acc = Op::ident();               // the single elements
+  uint32_t ws = 0;                         // offset of w's pieces from a 16-byte boundary
+  if constexpr (RAGGED) {
+    int64_t head = static_cast<int64_t>((16u - (reinterpret_cast<uintptr_t>(a + lo) & 15u)) & 15u) / static_cast<int64_t>(sizeof(E));
+    if (head > hi - lo) head = hi - lo;
+    int64_t body = (hi - lo - head) / kP * kP;
+    if constexpr (DOT) {
+      ws = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(w + lo + head) & 15u);
+      if (ws != 0 && body > 0 && lo + head < kP) {
+        head += kP;
+        body -= kP;
+      }
+      if (ws != 0 && body > 0 && lo + head + body + kP > R) body -= kP;
+    }
+    const int64_t first_end = lo + head, tail = lo + head + body;
+    for (int64_t x = t; x < (hi - lo) - body; x += T) {   // at most 15 + 16 elements on either side
+      const int64_t e = x < head ? lo + x : tail + (x - head);
+      const int32_t v = static_cast<int32_t>(a[e]);
+      if constexpr (OP == 0) {
+        acc = static_cast<int32_t>(static_cast<uint32_t>(acc) +
+                                   static_cast<uint32_t>(DOT ? v * static_cast<int32_t>(w[e]) : v));
+      } else {
+        acc = Op::combine(acc, v);
+      }
+    }
+    lo = first_end;
+    hi = tail;
+  }
+  const uint4* ap = reinterpret_cast<const uint4*>(a + lo) + t;
+  const uint4* wq = DOT ? reinterpret_cast<const uint4*>(w + lo - ws) + t : nullptr;
+  const int64_t pieces = (hi - lo) / kP;
+  int64_t n = t < pieces ? (pieces - t + T - 1) / T : 0;   // pieces of this thread
+  auto fold = [&](const uint4& q, const uint4& r) { Op::fold_piece(q, r, run, DOT); };
+  if (DOT && RAGGED && ws != 0) {
+    for (; n >= 2; n -= 2, ap += 2 * T, wq += 2 * T) {
+      const uint4 q0 = __ldcs(ap), q1 = __ldcs(ap + T);
+      const uint4 x0 = __ldg(wq), y0 = __ldg(wq + 1), x1 = __ldg(wq + T), y1 = __ldg(wq + T + 1);
+      fold(q0, shift_bytes(x0, y0, ws));
+      fold(q1, shift_bytes(x1, y1, ws));
+    }
+    if (n > 0) {
+      const uint4 q = __ldcs(ap);
+      fold(q, shift_bytes(__ldg(wq), __ldg(wq + 1), ws));
+    }
+  } else {
     for (; n >= 4; n -= 4, ap += 4 * T, wq += 4 * T) {       // four pieces in flight
       uint4 q[4], r[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         q[u] = __ldcs(ap + u * T);
         if constexpr (DOT) r[u] = __ldg(wq + u * T);
+        else r[u] = make_uint4(0u, 0u, 0u, 0u);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        Op::fold_word(q[u].x, DOT ? r[u].x : 0u, acc, pk, DOT);
-        Op::fold_word(q[u].y, DOT ? r[u].y : 0u, acc, pk, DOT);
-        Op::fold_word(q[u].z, DOT ? r[u].z : 0u, acc, pk, DOT);
-        Op::fold_word(q[u].w, DOT ? r[u].w : 0u, acc, pk, DOT);
-      }
+      for (int u = 0; u < 4; ++u) fold(q[u], r[u]);
     }
     for (; n > 0; --n, ap += T, wq += T) {
       const uint4 q = __ldcs(ap);
       uint4 r = make_uint4(0u, 0u, 0u, 0u);
       if constexpr (DOT) r = __ldg(wq);
-      Op::fold_word(q.x, r.x, acc, pk, DOT);
-      Op::fold_word(q.y, r.y, acc, pk, DOT);
-      Op::fold_word(q.z, r.z, acc, pk, DOT);
-      Op::fold_word(q.w, r.w, acc, pk, DOT);
-    }
-    if constexpr (OP != 0) acc = Op::unpack(pk);
-  } else {
-    for (int64_t x = lo + t; x < hi; x += T) {
-      const int32_t v = static_cast<int32_t>(a[x]);
-      if constexpr (OP == 0) {
-        acc = static_cast<int32_t>(static_cast<uint32_t>(acc) +
-                                   static_cast<uint32_t>(DOT ? v * static_cast<int32_t>(w[x]) : v));
-      } else {
-        acc = Op::combine(acc, v);
-      }
+      fold(q, r);
     }
   }
-  return acc;
+  return RAGGED ? Op::combine(acc, Op::value(run)) : Op::value(run);
 }
 
-// Teams of up to 256 threads are compiled for 8 resident CTAs per SM (32
-// registers): a streaming fold needs the bytes in flight of 2048 threads to
-// keep HBM busy.  Larger CTA teams (sub_width up to 32 warps) take a 1024-thread
-// variant.
-constexpr int kNarMinBlocks = 8;
-
-template <class E, int OP, bool DOT, bool VEC>
-__global__ void __launch_bounds__(kNarThreads, kNarMinBlocks) narrow_warp_kernel(NarArgs g) {
+template <class E, int OP, bool DOT, bool RAGGED>
+__global__ void __launch_bounds__(kNarThreads, RAGGED ? (DOT ? 5 : 6) : kNarMinBlocks) narrow_warp_kernel(NarArgs g) {
   using Op = NarrowOp<E, OP>;
   const int lane = threadIdx.x & 31;
   const int64_t warps = static_cast<int64_t>(gridDim.x) * (kNarThreads / 32);
   for (int64_t o = static_cast<int64_t>(blockIdx.x) * (kNarThreads / 32) + (threadIdx.x >> 5); o < g.O; o += warps) {
     const E* a = static_cast<const E*>(g.a) + o * g.R;
     const E* w = static_cast<const E*>(g.w);
-    int32_t v = fold_range<E, OP, DOT, VEC>(a, w, 0, g.R, lane, 32);
+    int32_t v = fold_range<E, OP, DOT, RAGGED>(a, w, 0, g.R, g.R, lane, 32);
     v = Op::warp_reduce(v);
     if (lane == 0) g.out[o] = v;
   }
 }
 
-template <class E, int OP, bool DOT, bool VEC, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == kNarThreads ? kNarMinBlocks : 1) narrow_block_kernel(NarArgs g) {
+template <class E, int OP, bool DOT, bool RAGGED, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == kNarThreads ? (RAGGED ? (DOT ? 5 : 6) : DOT ? kNarDotBlocks : kNarMinBlocks) : 1)
+    narrow_block_kernel(NarArgs g) {
   using Op = NarrowOp<E, OP>;
   __shared__ int32_t wp[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -277,7 +350,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == kNarThreads ? kNarMinBlocks : 1)
     const int64_t o = item / g.G, pg = item - o * g.G;
     const int64_t lo = pg * g.part_len, hi = std::min<int64_t>(lo + g.part_len, g.R);
     const E* a = static_cast<const E*>(g.a) + o * g.R;
-    int32_t v = fold_range<E, OP, DOT, VEC>(a, static_cast<const E*>(g.w), lo, hi, threadIdx.x, blockDim.x);
+    int32_t v = fold_range<E, OP, DOT, RAGGED>(a, static_cast<const E*>(g.w), lo, hi, g.R, threadIdx.x, blockDim.x);
     v = Op::warp_reduce(v);
     if (lane == 0) wp[warp] = v;
     __syncthreads();
@@ -303,6 +376,123 @@ __global__ void __launch_bounds__(MAXT, MAXT == kNarThreads ? kNarMinBlocks : 1)
   }
 }
 
+// Short rows: L lanes per row (short_lanes), 32 / L rows per warp and kShortRows
+// such sets in flight.  A row's first and last granule may hold
+// neighbouring rows' bytes: they are replaced by the identity (0 in a sum) with
+// masks from shared memory.  The dot product's w sits in shared memory in 16
+// copies, copy s shifted by s bytes, so that any alignment reads whole pieces.
+// Bound by instructions per granule (masks, shifts), by HBM for whole granules:
+// int8 sums of 268 MB, before (a warp per row, an element per load off 16-byte
+// boundaries) and now: 64-byte rows 376 and 44 us (6.5 TB/s), 333 bytes 109 and
+// 48, 500 bytes 125 and 54, 1000 bytes 118 and 45.
+constexpr int kShortBytes = 1024;             // rows off 16-byte boundaries
+constexpr int kShortAligned = 512;             // rows of whole granules (a warp per row of 1024 bytes reads 6.2 TB/s)
+constexpr int kShortRows = 4;
+constexpr int kShortW = kShortBytes + 48;   // one shifted copy of w, with the 16 bytes before and after it
+
+// a granule that reaches outside the array [first, last): its valid bytes [lo, hi) one by one
+__device__ __noinline__ uint4 granule_bytes(const unsigned char* p, int lo, int hi) {
+  uint32_t v[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    if (i >= lo && i < hi) v[i >> 2] |= static_cast<uint32_t>(p[i]) << (8 * (i & 3));
+  return make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+template <class E, int OP, bool DOT, bool RAGGED>
+__global__ void __launch_bounds__(kNarThreads, 4) narrow_rows_kernel(NarArgs g, int L) {
+  using Op = NarrowOp<E, OP>;
+  __shared__ __align__(16) uint32_t masks[RAGGED ? 256 : 1][4];   // bytes [lo, hi) of a granule: entry 16 lo + hi - 1
+  __shared__ __align__(16) uint32_t wcopy[DOT ? (RAGGED ? 16 : 1) : 1][DOT ? kShortW / 4 : 4];
+  const int tid = threadIdx.x;
+  if constexpr (RAGGED) {
+    for (int i = tid; i < 256 * 4; i += kNarThreads) {
+      const int word = i & 3, lo = i >> 6, hi = ((i >> 2) & 15) + 1;
+      uint32_t m = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (4 * word + k >= lo && 4 * word + k < hi) m |= 0xffu << (8 * k);
+      masks[i >> 2][word] = m;
+    }
+  }
+  if constexpr (DOT) {
+    const int n = static_cast<int>(g.R);
+    const unsigned char* wb = static_cast<const unsigned char*>(g.w);
+    constexpr int kWords = kShortW / 4;
+    for (int i = tid; i < (RAGGED ? 16 : 1) * kWords; i += kNarThreads) {
+      const int c = i / kWords, j = i - c * kWords;
+      uint32_t v = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int e = 4 * j + k + c - 16;                    // element of w at this byte
+        if (e >= 0 && e < n) v |= static_cast<uint32_t>(wb[e]) << (8 * k);
+      }
+      wcopy[c][j] = v;
+    }
+  }
+  __syncthreads();
+  const int lane = tid & 31, sub = lane & (L - 1), set = 32 / L;
+  const int row_bytes = static_cast<int>(g.R) * static_cast<int>(sizeof(E));
+  const int max_granules = RAGGED ? (row_bytes + 30) / 16 : row_bytes / 16;
+  const int64_t per_warp = static_cast<int64_t>(set) * kShortRows;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * (kNarThreads / 32) * per_warp;
+  int off[kShortRows];                                       // this lane's rows, in bytes from the warp's first
+#pragma unroll
+  for (int u = 0; u < kShortRows; ++u) off[u] = (u * set + lane / L) * row_bytes;
+  for (int64_t base = (static_cast<int64_t>(blockIdx.x) * (kNarThreads / 32) + (tid >> 5)) * per_warp; base < g.O;
+       base += stride) {
+    const unsigned char* const first = static_cast<const unsigned char*>(g.a) + base * row_bytes;
+    const int skew0 = static_cast<int>(reinterpret_cast<uintptr_t>(first) & 15u);
+    const int64_t left = g.O - base;
+    const bool ends = base == 0 || left <= per_warp + 15;    // a granule may reach outside the array
+    typename Op::Run run[kShortRows];
+    for (int j = sub; j < max_granules; j += L) {
+      uint4 q[kShortRows];
+      int lo[kShortRows], hi[kShortRows];                    // valid bytes of the granule
+#pragma unroll
+      for (int u = 0; u < kShortRows; ++u) {
+        const int skew = RAGGED ? (skew0 + off[u]) & 15 : 0;
+        const int at = off[u] - skew + 16 * j;
+        lo[u] = RAGGED && j == 0 ? skew : 0;
+        hi[u] = RAGGED ? min(16, row_bytes + skew - 16 * j) : 16;
+        if (ends && u * set + lane / L >= left) hi[u] = 0;
+        constexpr uint32_t id = Op::packed_ident();
+        q[u] = make_uint4(id, id, id, id);
+        if (hi[u] > 0) {
+          if (RAGGED && ends && (lo[u] > 0 || hi[u] < 16) &&
+              ((base == 0 && at < 0) || at + 16 > left * row_bytes))
+            q[u] = granule_bytes(first + at, lo[u], hi[u]);
+          else
+            q[u] = __ldcs(reinterpret_cast<const uint4*>(first + at));
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kShortRows; ++u) {
+        if constexpr (RAGGED) {
+          const uint4 m = *reinterpret_cast<const uint4*>(masks[16 * lo[u] + max(hi[u], 1) - 1]);
+          constexpr uint32_t id = Op::packed_ident();
+          q[u] = make_uint4((q[u].x & m.x) | (id & ~m.x), (q[u].y & m.y) | (id & ~m.y), (q[u].z & m.z) | (id & ~m.z),
+                            (q[u].w & m.w) | (id & ~m.w));
+        }
+        uint4 r = make_uint4(0u, 0u, 0u, 0u);
+        if constexpr (DOT) {
+          // the granule's first byte is element 16 j - skew; copies start 16 bytes before element 0
+          const int x = 16 * j + 16 - (RAGGED ? (skew0 + off[u]) & 15 : 0);
+          r = *reinterpret_cast<const uint4*>(&wcopy[RAGGED ? x & 15 : 0][(x >> 4) * 4]);
+        }
+        Op::fold_piece(q[u], r, run[u], DOT);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kShortRows; ++u) {
+      int32_t v = Op::value(run[u]);
+      for (int m = L >> 1; m >= 1; m >>= 1) v = Op::combine(v, __shfl_xor_sync(0xffffffffu, v, m));
+      const int row = u * set + lane / L;
+      if (sub == 0 && row < left) g.out[base + row] = v;
+    }
+  }
+}
+
 template <class K>
 int nar_blocks(K kernel, int threads, int sms) {
   int per = 0;
@@ -318,21 +508,44 @@ int64_t balanced_grid(int64_t items, int64_t resident) {
   return ceil_div64(items, waves);
 }
 
-template <class E, int OP, bool DOT, bool VEC>
+// lanes per short row: the fewest idle lane slots over at most four rounds of
+// granules, counting the reduction and the store as 2 log2 L + 6 of the about 40
+// instructions that a granule takes (500-byte rows: 16 lanes 102 us, 32 lanes,
+// half of them idle in the second round, 112)
+int short_lanes(int granules) {
+  int best = 32, cost = 1 << 30;
+  for (int lg = 5; lg >= 0; --lg) {
+    const int L = 1 << lg, rounds = (granules + L - 1) / L;
+    if (rounds > 4) break;
+    const int c = L * (40 * rounds + 2 * lg + 6);
+    if (c < cost) {
+      cost = c;
+      best = L;
+    }
+  }
+  return best;
+}
+
+template <class E, int OP, bool DOT, bool RAGGED>
 cudaError_t launch_narrow(const NarrowPlan& p, const NarArgs& g, int sms, cudaStream_t st) {
-  if (p.team == 0) {
+  if (p.team == 0 && p.R > 0 && p.R * p.esize <= (RAGGED ? kShortBytes : kShortAligned)) {
+    const int bytes = static_cast<int>(p.R) * p.esize;
+    const int L = short_lanes(RAGGED ? (bytes + 30) / 16 : bytes / 16);
+    auto k = narrow_rows_kernel<E, OP, DOT, RAGGED>;
+    const int64_t need = ceil_div64(p.O, static_cast<int64_t>(kNarThreads / L) * kShortRows);
+    k<<<static_cast<int>(balanced_grid(need, nar_blocks(k, kNarThreads, sms))), kNarThreads, 0, st>>>(g, L);
+  } else if (p.team == 0) {
     const int64_t need = ceil_div64(p.O, kNarThreads / 32);
-    const int grid =
-        static_cast<int>(balanced_grid(need, nar_blocks(narrow_warp_kernel<E, OP, DOT, VEC>, kNarThreads, sms)));
-    narrow_warp_kernel<E, OP, DOT, VEC><<<grid, kNarThreads, 0, st>>>(g);
+    auto k = narrow_warp_kernel<E, OP, DOT, RAGGED>;
+    k<<<static_cast<int>(balanced_grid(need, nar_blocks(k, kNarThreads, sms))), kNarThreads, 0, st>>>(g);
   } else {
     const int threads = 32 * p.W;
     if (threads <= kNarThreads) {
-      auto k = narrow_block_kernel<E, OP, DOT, VEC, kNarThreads>;
+      auto k = narrow_block_kernel<E, OP, DOT, RAGGED, kNarThreads>;
       const int grid = static_cast<int>(balanced_grid(p.O * p.G, nar_blocks(k, threads, sms)));
       k<<<grid, threads, 0, st>>>(g);
     } else {
-      auto k = narrow_block_kernel<E, OP, DOT, VEC, 1024>;
+      auto k = narrow_block_kernel<E, OP, DOT, RAGGED, 1024>;
       const int grid = static_cast<int>(balanced_grid(p.O * p.G, nar_blocks(k, threads, sms)));
       k<<<grid, threads, 0, st>>>(g);
     }
@@ -342,7 +555,7 @@ cudaError_t launch_narrow(const NarrowPlan& p, const NarArgs& g, int sms, cudaSt
 
 template <class E, int OP, bool DOT>
 cudaError_t launch_narrow_v(const NarrowPlan& p, const NarArgs& g, bool vec, int sms, cudaStream_t st) {
-  return vec ? launch_narrow<E, OP, DOT, true>(p, g, sms, st) : launch_narrow<E, OP, DOT, false>(p, g, sms, st);
+  return vec ? launch_narrow<E, OP, DOT, false>(p, g, sms, st) : launch_narrow<E, OP, DOT, true>(p, g, sms, st);
 }
 
 }  // namespace
