@@ -98,6 +98,7 @@ struct LaunchCfg {
   int cluster = 1;     // CTAs per cluster
   int combine_grid = 0;
   int M = 1;           // items per round of a block team
+  int rows = 0;        // the rows kernel this geometry is for (RowsKind; 0: none)
 };
 
 // Plan of a nest with an ordered (non-commutative) reduction: outputs over the

@@ -544,6 +544,298 @@ __global__ void __launch_bounds__(1024) rect_lanes_kernel(RectPlan p, Body body,
   }
 }
 
+// Reduce the partials of B items (part[r] = item r) over the L lanes of a
+// team in one go: recursive halving, each step handing half of the items to
+// the xor partner and combining the lower lane's partial first.  Every item
+// gets exactly the tree that lanes_allreduce builds at the team's lane 0, at
+// about one combine per item instead of log2(L).  On return part[0] of lane
+// lt holds item lt / (L / B) (B a power of two, B <= L).
+template <class Op, int B>
+__device__ __forceinline__ void lanes_reduce_many(typename Op::Acc (&part)[B], int L, int lt) {
+  using Acc = typename Op::Acc;
+  int m = L >> 1;
+#pragma unroll
+  for (int cnt = B; cnt > 1; cnt >>= 1, m >>= 1) {
+    const bool up = (lt & m) != 0;
+#pragma unroll
+    for (int i = 0; i < cnt / 2; ++i) {
+      const Acc send = up ? part[i] : part[i + cnt / 2];
+      const Acc keep = up ? part[i + cnt / 2] : part[i];
+      const Acc recv = Op::shfl_xor(send, m, L);
+      part[i] = up ? Op::combine(recv, keep) : Op::combine(keep, recv);
+    }
+  }
+  for (; m >= 1; m >>= 1) {
+    const Acc o = Op::shfl_xor(part[0], m, L);
+    part[0] = (lt & m) ? Op::combine(o, part[0]) : Op::combine(part[0], o);
+  }
+}
+constexpr int kReduceBatch = 4;   // items reduced together
+
+
+// ---------------------------------------------------------------- team = L lanes, whole rows
+// The plans that rect_lanes_kernel runs most, without its generality: one
+// reduced virtual level of stride 1 and no grid parts, so an output is a row of
+// R consecutive elements.  Every team folds U rows at once (row u of a warp's
+// set u) with U * NX row loads in flight; FP32 sums of one slot advance two rows
+// per packed FP32x2 instruction.  Each row sees the fold order and the reduction
+// tree of rect_lanes_kernel, so the bits are the same.  Bound by HBM for plain
+// sums (2^26 elements: rows of 64 and 1024, 51 and 47 us in the general kernel,
+// 41 here, 6.7 TB/s), by the compensated arithmetic's issue rate otherwise (dot
+// products of odd rows of 1021: 136 us, 72 here).
+struct RowsArgs {
+  int64_t O;
+  int32_t R, P, L;             // elements per row, slots (elements per step), lanes per team
+  int32_t grp_lanes, cg, cl;   // slot of lane lt: (lt / grp_lanes) * cg + (lt % grp_lanes) * cl
+};
+constexpr int kRowsThreads = 256;
+constexpr int64_t kRowsMaxR = int64_t(1) << 22;   // 32-bit offsets within a warp's rows
+
+// the U rows' values at one position, folded into their accumulators
+template <class Op, int V, bool DOT, int U>
+__device__ __forceinline__ void fold_rows(typename Op::Acc (&acc)[U][V], const Vals<Op, V> (&v)[U],
+                                          const typename Op::In (&b)[V]) {
+  if constexpr (V == 1 && U % 2 == 0 && std::is_same<Op, OpF32Comp>::value) {
+#pragma unroll
+    for (int u = 0; u < U; u += 2) {
+      float2 sp = make_float2(acc[u][0].s, acc[u + 1][0].s), cp = make_float2(acc[u][0].c, acc[u + 1][0].c);
+      const float2 x = make_float2(v[u].a[0], v[u + 1].a[0]);
+      if constexpr (DOT) comp_prod_pair(sp, cp, x, make_float2(b[0], b[0]));
+      else comp_add_pair(sp, cp, x);
+      acc[u][0] = {sp.x, cp.x};
+      acc[u + 1][0] = {sp.y, cp.y};
+    }
+  } else if constexpr (V == 1 && U % 2 == 0 && std::is_same<Op, OpF32Sum>::value) {
+#pragma unroll
+    for (int u = 0; u < U; u += 2) {
+      float2 sp = make_float2(acc[u][0], acc[u + 1][0]);
+      const float2 x = make_float2(v[u].a[0], v[u + 1].a[0]);
+      if constexpr (DOT) sp = fma2(x, make_float2(b[0], b[0]), sp);
+      else sp = add2(sp, x);
+      acc[u][0] = sp.x;
+      acc[u + 1][0] = sp.y;
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if constexpr (DOT) fold_vals_dot<Op, V>(acc[u], v[u].a, b);
+      else fold_vals_load<Op, V>(acc[u], v[u].a);
+    }
+  }
+}
+template <class In, int V>
+__device__ __forceinline__ void load_row(const In* p, In (&a)[V]) {
+  if constexpr (V == 4) {
+    const auto q = ld_stream4(p);
+    a[0] = q.x;
+    a[1] = q.y;
+    a[2] = q.z;
+    a[3] = q.w;
+  } else {
+    a[0] = ld_stream(p);
+  }
+}
+template <class In, int V>
+__device__ __forceinline__ void load_bcast(const In* p, In (&b)[V]) {
+  if constexpr (V == 4) {
+    const auto q = ld_keep4(p);
+    b[0] = q.x;
+    b[1] = q.y;
+    b[2] = q.z;
+    b[3] = q.w;
+  } else {
+    b[0] = ld_keep(p);
+  }
+}
+// A team folds one row at a time with 4 positions loaded ahead: the registers
+// that more rows take cost more resident warps than their loads are worth.  A
+// thread per row of at most 4 elements has no further positions: 4 rows.
+constexpr int kRowsU = 4;
+
+// CTAs per SM the registers are sized for (swept over 5, 6 and 8, and uncapped):
+// 2^26 elements in rows of 100 / 511, f32: 6 and 8 CTAs 43 and 48 us, uncapped 45
+// and 55; compensated dot: 57 and 70 us, uncapped 77 and 73
+template <class Op, int V, bool DOT, int U>
+constexpr int rows_blocks() {
+  if (U > 1) return 1;
+  if (V == 1) return 8;
+  return !DOT && sizeof(typename Op::Acc) == 8 ? 5 : 6;
+}
+
+template <class Op, int V, bool DOT, int U>
+__global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
+    rect_rows_kernel(const RowsArgs g, const typename Op::In* __restrict__ A, const typename Op::In* __restrict__ w,
+                     typename Op::Out* out, float* comp) {
+  using Acc = typename Op::Acc;
+  using In = typename Op::In;
+  constexpr int NX = U == 1 ? 4 : 2;            // positions loaded before the first fold
+  const int L = g.L, R = g.R, P = g.P;
+  const int lane = threadIdx.x & 31, lt = lane & (L - 1), set = 32 / L;
+  const int s0 = (lt / g.grp_lanes) * g.cg + (lt % g.grp_lanes) * g.cl;
+  const int64_t per = static_cast<int64_t>(set) * U;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5) * per;
+  for (int64_t base = (static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per; base < g.O;
+       base += stride) {
+    const int64_t row = base + lane / L;
+    const In* a = A + row * R;
+    const int dist = set * R;                   // elements between a team's rows
+    Acc acc[U][V];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int i = 0; i < V; ++i) acc[u][i] = Op::ident();
+    const bool whole = base + per <= g.O;       // the same in every lane
+    int rows = U;                               // this lane's rows
+    if (!whole) {
+      rows = 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) rows += row + static_cast<int64_t>(u) * set < g.O ? 1 : 0;
+    }
+    int x = s0;
+    if (whole) {
+      for (; x + (NX - 1) * P < R; x += NX * P) {
+        Vals<Op, V> v[NX][U];
+        In b[NX][V];
+#pragma unroll
+        for (int q = 0; q < NX; ++q) {
+          if constexpr (DOT) load_bcast<In, V>(w + x + q * P, b[q]);
+#pragma unroll
+          for (int u = 0; u < U; ++u) load_row<In, V>(a + u * dist + x + q * P, v[q][u].a);
+        }
+#pragma unroll
+        for (int q = 0; q < NX; ++q) fold_rows<Op, V, DOT, U>(acc, v[q], b[q]);
+      }
+    }
+    for (; x < R; x += P) {
+      Vals<Op, V> v[U];
+      In b[V];
+      if constexpr (DOT) load_bcast<In, V>(w + x, b);
+      // rows past the last are folded from the first row's values; their results are not stored
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (rows > 0) load_row<In, V>(a + (u < rows ? u * dist : 0) + x, v[u].a);
+      if (rows > 0) fold_rows<Op, V, DOT, U>(acc, v, b);
+    }
+    Acc part[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) part[u] = fold_vec<Op, V>(acc[u]);
+    if (U > 1 && L >= U) {
+      lanes_reduce_many<Op, U>(part, L, lt);
+      const int64_t o = row + static_cast<int64_t>(lt / (L / U)) * set;
+      if ((lt & (L / U - 1)) == 0 && o < g.O) {
+        out[o] = Op::finish(part[0]);
+        if constexpr (std::is_same_v<Acc, f2>) {
+          if (comp) comp[o] = Op::residual(part[0]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const Acc r = lanes_allreduce<Op>(part[u], L);
+        const int64_t o = row + static_cast<int64_t>(u) * set;
+        if (lt == 0 && o < g.O) {
+          out[o] = Op::finish(r);
+          if constexpr (std::is_same_v<Acc, f2>) {
+            if (comp) comp[o] = Op::residual(r);
+          }
+        }
+      }
+    }
+  }
+}
+
+// Teams of one lane (rows of 5 to 32 elements) or two (odd rows of up to 64): the
+// rows of a warp's teams are one contiguous block, so the warp copies it to
+// shared memory with 16-byte cp.async (its stage ring keeps the next two blocks
+// in flight) and the teams fold their rows from there.  Read straight from global
+// memory, such a row takes a sector per team and load: 2^26 elements in rows of
+// 31, f32, 135 us so, 51 here.
+constexpr int kThreadRowsMin = 5, kThreadRowsMax = 64;
+constexpr int kThreadRowsStages = 3;
+
+template <class Op, int V, bool DOT>
+__global__ void __launch_bounds__(kRowsThreads) rect_thread_rows_kernel(int64_t O, int R, int L,
+                                                                        const typename Op::In* __restrict__ A,
+                                                                        const typename Op::In* __restrict__ w,
+                                                                        typename Op::Out* out, float* comp) {
+  using Acc = typename Op::Acc;
+  using In = typename Op::In;
+  extern __shared__ __align__(16) unsigned char rows_smem[];
+  __shared__ __align__(16) In ws[DOT ? kThreadRowsMax : 4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if constexpr (DOT) {
+    if (static_cast<int>(threadIdx.x) < R) ws[threadIdx.x] = w[threadIdx.x];
+    __syncthreads();
+  }
+  const int set = 32 / L;
+  const int block = set * R;                     // elements of a block; 64 R or 128 R bytes, so blocks keep A's alignment
+  In* const ring = reinterpret_cast<In*>(rows_smem) + warp * kThreadRowsStages * block;
+  const int64_t n_blocks = (O + set - 1) / set;
+  const int64_t first = static_cast<int64_t>(blockIdx.x) * (kRowsThreads / 32) + warp;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * (kRowsThreads / 32);
+  auto issue = [&](int64_t b, int stage) {
+    if (b < n_blocks) {
+      const int64_t left = (O - b * set) * R;    // elements of A from the block on
+      const In* src = A + b * set * R;
+      for (int i = 4 * lane; i < block; i += 128) {
+        const int n = left - i >= 4 ? 4 : left > i ? static_cast<int>(left - i) : 0;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(ring + stage * block + i)),
+                     "l"(n > 0 ? src + i : A), "r"(4 * n)
+                     : "memory");
+      }
+    }
+    cp_async_commit();
+  };
+  int64_t next = first;
+#pragma unroll
+  for (int s = 0; s < kThreadRowsStages - 1; ++s, next += stride) issue(next, s);
+  int stage = 0, refill = kThreadRowsStages - 1;
+  for (int64_t b = first; b < n_blocks; b += stride, next += stride) {
+    cp_async_wait<kThreadRowsStages - 2>();
+    __syncwarp();                                // every lane's copies; and every lane has read the stage refilled below
+    issue(next, refill);
+    const int lt = lane & (L - 1);
+    const In* row = ring + stage * block + lane / L * R;
+    refill = stage;
+    stage = stage + 1 == kThreadRowsStages ? 0 : stage + 1;
+    Acc acc[1][V];
+#pragma unroll
+    for (int i = 0; i < V; ++i) acc[0][i] = Op::ident();
+    for (int x = V * lt; x < R; x += V * L) {
+      Vals<Op, V> v[1];
+      In bb[V];
+      if constexpr (V == 4) {
+        using V4 = typename Vec4Of<In>::T;
+        const V4 q = *reinterpret_cast<const V4*>(row + x);
+        v[0].a[0] = q.x;
+        v[0].a[1] = q.y;
+        v[0].a[2] = q.z;
+        v[0].a[3] = q.w;
+        if constexpr (DOT) {
+          const V4 t = *reinterpret_cast<const V4*>(ws + x);
+          bb[0] = t.x;
+          bb[1] = t.y;
+          bb[2] = t.z;
+          bb[3] = t.w;
+        }
+      } else {
+        v[0].a[0] = row[x];
+        if constexpr (DOT) bb[0] = ws[x];
+      }
+      fold_rows<Op, V, DOT, 1>(acc, v, bb);
+    }
+    const int64_t o = b * set + lane / L;
+    const Acc t = lanes_allreduce<Op>(fold_vec<Op, V>(acc[0]), L);
+    if (lt == 0 && o < O) {
+      out[o] = Op::finish(t);
+      if constexpr (std::is_same_v<Acc, f2>) {
+        if (comp) comp[o] = Op::residual(t);
+      }
+    }
+  }
+  cp_async_wait<0>();
+}
+
 // ---------------------------------------------------------------- grid parts -> outputs
 // A warp per output: the lanes stage up to 256 parts at a time in shared
 // memory with coalesced loads, and lane 0 folds them in part order (the steps

@@ -26,6 +26,63 @@ inline hp_status cuda_fail(cudaError_t e, const char* what) {
   return fail(HP_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// Which kernel folds whole rows (rect_rows_kernel, rect_thread_rows_kernel)?
+enum RowsKind { ROWS_NONE = 0, ROWS_TEAM = 1, ROWS_THREAD = 2 };
+inline RowsKind rows_kind(const RectPlan& rp, const void* A) {
+  if (rp.team != TEAM_LANES || rp.nv != 1 || rp.vstride[0] != 1 || rp.G != 1 || rp.split || rp.R < 1 || rp.R > kRowsMaxR)
+    return ROWS_NONE;
+  // one or two lanes a row: blocks of 32 rows are copied 16 bytes at a time
+  const bool aligned = (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
+  if (rp.R >= kThreadRowsMin && aligned && rp.cl[0] == rp.V &&
+      (rp.L == 1 ? rp.R <= 32 : rp.L == 2 && rp.V == 1 && rp.grp_lanes >= 2 && rp.R <= kThreadRowsMax))
+    return ROWS_THREAD;
+  return rp.L > 1 || rp.R < kThreadRowsMin ? ROWS_TEAM : ROWS_NONE;
+}
+
+// launch of a rows kernel; cfg is filled on the nest's first run of that kind
+template <class Op, int V, bool DOT>
+hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const typename Op::In* A,
+                      const typename Op::In* w, const RectArgs& a) {
+  using Out = typename Op::Out;
+  auto k1 = rect_rows_kernel<Op, V, DOT, 1>;
+  auto k4 = rect_rows_kernel<Op, V, DOT, kRowsU>;
+  auto kt = rect_thread_rows_kernel<Op, V, DOT>;
+  const int set = 32 / rp.L;
+  const size_t dyn = kind == ROWS_THREAD ? sizeof(int32_t) * (kRowsThreads / 32) * kThreadRowsStages * set * rp.R : 0;
+  const int U = rp.L == 1 ? kRowsU : 1;
+  if (!cfg.ready || cfg.rows != kind) {
+    const void* f = kind == ROWS_THREAD ? reinterpret_cast<const void*>(kt)
+                    : U == 1            ? reinterpret_cast<const void*>(k1)
+                                        : reinterpret_cast<const void*>(k4);
+    cudaError_t e = cudaSuccess;
+    if (kind == ROWS_THREAD)   // the kernel's largest, whatever this nest needs
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kRowsThreads / 32 * kThreadRowsStages * 4 * 32 * 32);
+    if (e != cudaSuccess) return cuda_fail(e, "dynamic shared memory size");
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kRowsThreads, dyn);
+    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    if (per_sm < 1) return fail(HP_EUNSUPPORTED, "kernel does not fit on an SM with this CTA size");
+    const int64_t cta_rows = static_cast<int64_t>(kRowsThreads / 32) * set * (kind == ROWS_THREAD ? 1 : U);
+    const int64_t blocks = std::min<int64_t>((rp.O + cta_rows - 1) / cta_rows, static_cast<int64_t>(per_sm) * cfg.sms);
+    cfg.threads = kRowsThreads;
+    cfg.grid = static_cast<int>(std::max<int64_t>(blocks, 1));
+    cfg.rows = kind;
+    cfg.ready = true;
+  }
+  if (rp.O == 0) return HP_OK;
+  Out* out = static_cast<Out*>(a.out);
+  if (kind == ROWS_THREAD) {
+    kt<<<cfg.grid, kRowsThreads, dyn, a.stream>>>(rp.O, static_cast<int>(rp.R), rp.L, A, w, out, a.comp);
+  } else {
+    const RowsArgs g{rp.O, static_cast<int32_t>(rp.R), rp.vP[0], rp.L, rp.grp_lanes, rp.cg[0], rp.cl[0]};
+    if (U == 1) k1<<<cfg.grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
+    else k4<<<cfg.grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
+  }
+  const cudaError_t e = cudaPeekAtLastError();
+  return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_rows_kernel launch");
+}
+
 template <class Op, int V, class Body>
 hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Body& body, const RectArgs& a) {
   using Out = typename Op::Out;
@@ -45,6 +102,10 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
     e = cudaPeekAtLastError();
     return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_map_kernel launch");
   }
+  if constexpr (Body::kPipeable) {
+    const RowsKind kind = rows_kind(rp, body.A);
+    if (kind != ROWS_NONE) return launch_rows<Op, V, Body::kDot>(rp, kind, cfg, body.A, body.wptr(), a);
+  }
   const bool block = rp.team == TEAM_BLOCK;
   constexpr bool kPipeable = Body::kPipeable && V == 4;
   const bool pipe = kPipeable && block && rp.pipe;
@@ -58,7 +119,8 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
       pipe ? static_cast<size_t>(32 * rp.W) *
                  std::max<size_t>(pipe_depth(rp.groups) * rp.groups * 16, kPatMax * sizeof(int32_t))
            : 0;
-  if (!cfg.ready) {
+  if (!cfg.ready || cfg.rows != ROWS_NONE) {
+    cfg.rows = ROWS_NONE;
     cfg.threads = 32 * rp.W;
     cfg.cluster = block ? rp.C : 1;
     if (pipe) {
