@@ -387,30 +387,39 @@ __device__ __forceinline__ long long ld_part(const long long* p) { return __ldcg
 
 // The final combine of one output's G partials (the second pass of Sec. 2's
 // recursive reduction when a reduced level is split over the grid), shared by
-// every executor so that their results agree bit for bit.  Parts are folded
-// in part order.  Compensated partials (s_g, c_g) are added as double-float
-// numbers: TwoSum carries s_g into the running sum exactly, and its error and
-// c_g go to a second FP32 word (the cascaded summation of Ogita, Rump and
-// Oishi, "Accurate sum and dot product", 2005); the result is the rounded sum
-// of the two words and rem (may be null) its exact rounding error.  Its error
-// is at most gamma_2G (gamma_G + 2 gamma_k) sum|t| beyond the parts' own (k
-// the parts' chain length), far below the FP32 result's rounding.  FP64 is
-// not used: a dependent FP64 operation costs about 63 SM cycles on this GPU
-// (FP32: 4.5), and a chain of 2G of them took about 40 us for G = 304.
-// one fold step of that combine; every executor folds the same steps in the
-// same order
+// every executor so that their results agree bit for bit.  Part g belongs to
+// chain g mod 32; every chain folds its parts in order, and the chains combine
+// in a butterfly (neighbours first, the lower chain's value on the left).  One
+// chain over all parts was a third of a single-output run: 608 dependent
+// TwoSums take about 10 us.  Compensated partials (s_g, c_g) are added as
+// double-float numbers: TwoSum carries s_g into the running sum exactly, and
+// its error and c_g go to a second FP32 word (the cascaded summation of Ogita,
+// Rump and Oishi, "Accurate sum and dot product", 2005); the result is the
+// rounded sum of the two words and rem (may be null) its exact rounding error.
+// Its error is at most gamma_2G (gamma_G + 2 gamma_k) sum|t| beyond the parts'
+// own (k the parts' chain length; the bound of one chain over all parts, which
+// the 32 shorter ones stay below), far below the FP32 result's rounding.  FP64
+// is not used: a dependent FP64 operation costs about 63 SM cycles on this GPU
+// (FP32: 4.5).
+constexpr int kPartChains = 32;
 template <class Op, bool COMP = std::is_same_v<typename Op::Acc, f2>>
 struct PartFold;
 template <class Op>
 struct PartFold<Op, true> {
   float S = 0.0f, C = 0.0f;
-  __device__ __forceinline__ void first(const f2& v) { add(v); }
   __device__ __forceinline__ void add(const f2& v) {
     float s2, e;
     two_sum(S, v.s, s2, e);
     S = s2;
     C = __fadd_rn(C, e);
     C = __fadd_rn(C, v.c);
+  }
+  __device__ __forceinline__ void merge(const PartFold& b) { add(f2{b.S, b.C}); }   // another chain's value, on the right
+  __device__ __forceinline__ PartFold shfl_xor(int m) const {
+    PartFold r;
+    r.S = __shfl_xor_sync(0xffffffffu, S, m);
+    r.C = __shfl_xor_sync(0xffffffffu, C, m);
+    return r;
   }
   __device__ __forceinline__ float result(float* rem) const {
     float r, e;
@@ -421,29 +430,80 @@ struct PartFold<Op, true> {
 };
 template <class Op>
 struct PartFold<Op, false> {
-  typename Op::Acc a;
-  __device__ __forceinline__ void first(const typename Op::Acc& v) { a = v; }
+  typename Op::Acc a = Op::ident();
   __device__ __forceinline__ void add(const typename Op::Acc& v) { a = Op::combine(a, v); }
+  __device__ __forceinline__ void merge(const PartFold& b) { a = Op::combine(a, b.a); }
+  __device__ __forceinline__ PartFold shfl_xor(int m) const {
+    PartFold r;
+    r.a = Op::shfl_xor(a, m, 32);
+    return r;
+  }
   __device__ __forceinline__ typename Op::Out result(float*) const { return Op::finish(a); }
 };
 
-// the combine by one thread, loading 8 parts at a time from L2
+// the combine by one thread: eight chains at a time, eight parts in flight.
+// A chain without parts holds the identity, and merging it changes nothing (the
+// sums start from +0, so no chain holds -0): groups past G are left out.
 template <class Op>
 __device__ __forceinline__ typename Op::Out combine_parts(const typename Op::Acc* pp, int32_t G, float* rem) {
   using Acc = typename Op::Acc;
   constexpr int K = 8;
-  PartFold<Op> f;
-  f.first(ld_part(pp));
-  int32_t g = 1;
-  for (; g + K <= G; g += K) {
-    Acc v[K];
+  PartFold<Op> out, pair;   // chains 0 .. 15 and all; the current 16 chains
+#pragma unroll 1
+  for (int32_t c0 = 0; c0 < kPartChains && c0 < G; c0 += K) {
+    PartFold<Op> f[K];
+    int32_t g = c0;
+#pragma unroll 1
+    for (; g + K <= G; g += kPartChains) {
+      Acc v[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = ld_part(pp + g + k);
+      for (int k = 0; k < K; ++k) v[k] = ld_part(pp + g + k);
 #pragma unroll
-    for (int k = 0; k < K; ++k) f.add(v[k]);
+      for (int k = 0; k < K; ++k) f[k].add(v[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < K - 1; ++k)
+      if (g + k < G) f[k].add(ld_part(pp + g + k));
+#pragma unroll
+    for (int m = 1; m < K; m <<= 1)
+#pragma unroll
+      for (int k = 0; k < K; k += 2 * m) f[k].merge(f[k + m]);
+    if (c0 & K) pair.merge(f[0]);
+    else pair = f[0];
+    if ((c0 & K) || c0 + K >= G) {
+      if (c0 < 2 * K) out = pair;
+      else out.merge(pair);
+    }
   }
-  for (; g < G; ++g) f.add(ld_part(pp + g));
-  return f.result(rem);
+  return out.result(rem);
+}
+
+// the same by a warp, a chain per lane; lane 0 has the result
+template <class Op>
+__device__ __forceinline__ typename Op::Out combine_parts_warp(const typename Op::Acc* pp, int32_t G, int lane,
+                                                               float* rem) {
+  using Acc = typename Op::Acc;
+  PartFold<Op> f;
+  int32_t g = lane;
+  for (; g + 3 * kPartChains < G; g += 4 * kPartChains) {
+    Acc v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = ld_part(pp + g + k * kPartChains);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f.add(v[k]);
+  }
+  for (; g < G; g += kPartChains) f.add(ld_part(pp + g));
+#pragma unroll
+  for (int m = 1; m < kPartChains; m <<= 1) {
+    PartFold<Op> o = f.shfl_xor(m);
+    if (lane & m) {
+      o.merge(f);
+      f = o;
+    } else {
+      f.merge(o);
+    }
+  }
+  return f.result(lane == 0 ? rem : nullptr);
 }
 
 }  // namespace hp

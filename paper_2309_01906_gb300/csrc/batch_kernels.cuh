@@ -123,34 +123,41 @@ struct EmitTo {
   int32_t G;
 };
 
-// the last part of an output to arrive combines them all (the combine of
-// rect_combine_kernel, so results equal hp_nest_run's); out of line, so that
-// its registers do not weigh on the streaming loops that call batch_emit
+// A warp emits its items, lane l's if `valid` (every lane calls).  The last part
+// of an output to arrive combines them all, a chain of parts per lane: the
+// combine of rect_combine_kernel, so results equal hp_nest_run's.  (One thread
+// folding every part took its registers from the streaming loops around it.)
 template <class Op>
-__device__ __forceinline__ void batch_combine(const typename Op::Acc* pp, int32_t G, typename Op::Out* out) {
-  *out = combine_parts<Op>(pp, G, nullptr);
-}
-
-template <class Op>
-__device__ __forceinline__ void batch_emit(const EmitTo& to, int64_t item, typename Op::Acc a) {
+__device__ __forceinline__ void batch_emit(const EmitTo& to, int64_t item, typename Op::Acc a, bool valid, int lane) {
   using Acc = typename Op::Acc;
   if (to.G == 1) {
-    static_cast<typename Op::Out*>(to.out)[item] = Op::finish(a);
+    if (valid) static_cast<typename Op::Out*>(to.out)[item] = Op::finish(a);
     return;
   }
   Acc* part = static_cast<Acc*>(to.part);
   const int64_t o = item / to.G;
-  part[item] = a;
-  __threadfence();  // publish the partial before taking the ticket
-  if (atomicAdd(&to.tickets[o], 1) == to.G - 1) {
+  bool mine = false;
+  if (valid) {
+    part[item] = a;
+    __threadfence();  // publish the partial before taking the ticket
+    mine = atomicAdd(&to.tickets[o], 1) == to.G - 1;
+  }
+  unsigned last = __ballot_sync(0xffffffffu, mine);
+  while (last) {
+    const int64_t oc = __shfl_sync(0xffffffffu, o, __ffs(last) - 1);
+    last &= last - 1;
     __threadfence();  // all parts of this output are visible
-    batch_combine<Op>(part + o * to.G, to.G, static_cast<typename Op::Out*>(to.out) + o);
-    to.tickets[o] = 0;  // ready for the next run
+    const typename Op::Out r = combine_parts_warp<Op>(part + oc * to.G, to.G, lane, nullptr);
+    if (lane == 0) {
+      static_cast<typename Op::Out*>(to.out)[oc] = r;
+      to.tickets[oc] = 0;  // ready for the next run
+    }
   }
 }
 template <class Op>
-__device__ __forceinline__ void batch_emit(const RectPlan& p, const BatchNest& bn, int64_t item, typename Op::Acc a) {
-  batch_emit<Op>(EmitTo{bn.out, bn.part, bn.tickets, p.G}, item, a);
+__device__ __forceinline__ void batch_emit(const RectPlan& p, const BatchNest& bn, int64_t item, typename Op::Acc a,
+                                           bool valid, int lane) {
+  batch_emit<Op>(EmitTo{bn.out, bn.part, bn.tickets, p.G}, item, a, valid, lane);
 }
 
 // ---------------------------------------------------------------- mbarrier / bulk-copy primitives
@@ -439,10 +446,10 @@ __device__ __forceinline__ void batch_block_items(const RectPlan& p, const Body&
     const Acc a = lanes_allreduce<Op>(fold_vec<Op, V>(acc), 32);
     if (lane == 0 && active) wsh[warp] = a;
     consumer_sync();
-    if (tid == 0) {
+    if (warp == 0) {
       Acc r = wsh[0];
       for (int w = 1; w < p.W; ++w) r = Op::combine(r, wsh[w]);
-      batch_emit<Op>(p, bn, item, r);
+      batch_emit<Op>(p, bn, item, r, lane == 0, lane);
     }
     consumer_sync();
   }
@@ -473,7 +480,7 @@ __device__ __forceinline__ void batch_lanes_items(const RectPlan& p, const Body&
       fold_item<Op, V>(p, body, o, g, slot, acc);
     }
     const Acc a = lanes_allreduce<Op>(fold_vec<Op, V>(acc), L);
-    if (valid && lt == 0) batch_emit<Op>(p, bn, item, a);
+    batch_emit<Op>(p, bn, item, a, valid && lt == 0, lane);
   }
 }
 
@@ -573,10 +580,13 @@ __device__ __forceinline__ void ring_block_items(const RingGeom& gm, const Fold&
       if ((lane & (32 / kReduceBatch - 1)) == 0 && active && mb + k < mc) wsh[buf][mb + k][warp] = part[0];
     }
     consumer_sync();
-    if (tid < mc) {
-      Acc r = wsh[buf][tid][0];
-      for (int w = 1; w < W; ++w) r = Op::combine(r, wsh[buf][tid][w]);
-      batch_emit<Op>(bn.rp, bn, item0 + m0 + tid, r);
+    if (warp == 0) {   // a chunk's items: at most one per lane
+      Acc r = Op::ident();
+      if (lane < mc) {
+        r = wsh[buf][lane][0];
+        for (int w = 1; w < W; ++w) r = Op::combine(r, wsh[buf][lane][w]);
+      }
+      batch_emit<Op>(EmitTo{bn.out, bn.part, bn.tickets, gm.G}, item0 + m0 + lane, r, lane < mc, lane);
     }
   }
 }
@@ -666,7 +676,7 @@ __device__ __forceinline__ void ring_lanes_items(const RingGeom& gm, const Fold&
         fold.template run<V>(base + lo, lo, s0, static_cast<int32_t>(hi - lo), gm.P, acc);
       }
       const Acc a = lanes_allreduce<Op>(fold_vec<Op, V>(acc), L);
-      if (valid && lt == 0) batch_emit<Op>(bn.rp, bn, item0 + b + j, a);
+      batch_emit<Op>(bn.rp, bn, item0 + b + j, a, valid && lt == 0, tid & 31);
     }
     ring_release(rv, ring_stage(rv, w_end), rel);
   }

@@ -96,7 +96,6 @@ struct LaunchCfg {
   int grid = 0;        // CTAs
   int threads = 0;     // per CTA
   int cluster = 1;     // CTAs per cluster
-  int combine_grid = 0;
   int M = 1;           // items per round of a block team
   int rows = 0;        // the rows kernel this geometry is for (RowsKind; 0: none)
 };

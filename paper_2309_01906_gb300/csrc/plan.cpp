@@ -109,6 +109,33 @@ size_t tune_cache_size() {
   return g_tune.size();
 }
 
+// Grid parts per output for O outputs of n iterations, with parts of at least
+// kMinPart (a part's reduction tree and its place in the combine cost about as
+// much as folding a few thousand iterations): the fewest that give every SM
+// HP_PLAN_TEAMS_PER_SM teams with no SM more than a twentieth behind the others,
+// else the most even ones.  Two teams per SM left a 1 GiB single-output sum at
+// 3.7 TB/s, four reach 5.7; 640 teams (4.2 per SM) ran at the pace of 5 per SM.
+static int64_t grid_parts(int64_t O, int64_t n) {
+  const int64_t most = std::max<int64_t>(1, n / kMinPart);
+  if (O < 1) return 1;
+  int64_t best = 1;
+  double best_even = -1.0;
+  for (int64_t G = 1; G <= most; ++G) {
+    const int64_t items = O * G, per_sm = (items + kAssumedSMs - 1) / kAssumedSMs;
+    if (items < HP_PLAN_TEAMS_PER_SM * kAssumedSMs) {
+      best = G;          // too few teams: as many as there are
+      continue;
+    }
+    const double even = static_cast<double>(items) / static_cast<double>(per_sm * kAssumedSMs);
+    if (even > best_even) {
+      best_even = even;
+      best = G;
+    }
+    if (even >= 0.95 || items > 32 * kAssumedSMs) break;
+  }
+  return best;
+}
+
 static void auto_map(const NestPlan& p, hp_level_map* m);
 
 // outputs over the grid; every reduced level on the chosen hardware level
@@ -162,7 +189,7 @@ static void auto_map(const NestPlan& p, hp_level_map* m) {
   int red_hw;
   int sub = 0;
   if (R >= 4096) {
-    red_hw = (O < 2 * kAssumedSMs && R >= 65536) ? HP_HW_GRID : HP_HW_CTA;
+    red_hw = (O < 12 * kAssumedSMs && R >= 65536 && grid_parts(O, R) > 1) ? HP_HW_GRID : HP_HW_CTA;
   } else if (R >= 512) {
     red_hw = HP_HW_WARP;
   } else if (R >= 32) {
@@ -423,13 +450,8 @@ hp_status plan_rect(int depth, const int64_t* extents, const hp_level_map* map, 
     for (int l = vls[0].first; l <= vls[0].last; ++l)
       if (m[l].tile > 0) tile = m[l].tile;
     if (tile <= 0) {
-      // aim at about four block teams per SM over all outputs (two left a
-      // 1 GiB single-output sum at 3.7 TB/s, four reach 5.7), with parts of
-      // at least kMinPart iterations (a part's reduction tree and its ticket
-      // cost about as much as folding a few thousand iterations)
-      const int64_t teams = HP_PLAN_TEAMS_PER_SM * kAssumedSMs;
-      int64_t want_parts = std::max<int64_t>(1, (teams + O - 1) / std::max<int64_t>(O, 1));
-      want_parts = std::min<int64_t>(want_parts, std::max<int64_t>(1, n0 / kMinPart));
+      tile = 0;
+      const int64_t want_parts = grid_parts(O, n0);
       tile = (n0 + want_parts - 1) / std::max<int64_t>(want_parts, 1);
     }
     if (nv == 1 && V > 1) tile = (tile + V - 1) / V * V;

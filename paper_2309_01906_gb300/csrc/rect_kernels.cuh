@@ -12,8 +12,8 @@
 //                      Sec. 3.8, or a single thread): lanes combine by
 //                      xor-shuffle with width L.
 // When the first reduced level is bound to the grid, every output is cut into
-// G parts that write partials; rect_combine_kernel folds them in part order
-// (combine_parts; compensated partials as a double-float sum).
+// G parts that write partials; rect_combine_kernel folds them in 32 interleaved
+// chains (accum.cuh; compensated partials as a double-float sum).
 // The reduction tree depends only on the plan, never on which SM ran what, so
 // runs are bit-reproducible.
 #pragma once
@@ -744,6 +744,91 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
   }
 }
 
+// ---------------------------------------------------------------- team = a CTA, contiguous items
+// The plans of rect_block_kernel with one reduced virtual level of stride 1 and
+// a CTA of at most 8 warps: an item (an output, or one grid part of it) is a run
+// of consecutive elements.  The per-thread order and the tree are
+// rect_block_kernel's; what differs is what limits the rate: 32-bit offsets, no
+// general level loop and 256 threads a CTA leave 32 to 48 registers a thread, so
+// 4 to 8 CTAs per SM keep 4 or 8 loads per thread in flight.  2^26 elements in
+// rows of 16384, 262144 and one row, f32: 45, 61 and 54 us in the general kernel,
+// 39, 44 and 47 here (6.9 TB/s; the single row adds its combine's launch); odd
+// rows of 8195: 73 and 41; compensated dot of 16384: 69 and 43.
+struct FlatArgs {
+  int64_t items, R, tile;      // tile: elements per grid part (G > 1)
+  int32_t G, P, W;
+  int32_t grp_lanes, cw, cg, cl;
+};
+constexpr int kFlatThreads = 256;
+// CTAs per SM (swept): the dot product's second operand takes the registers of
+// one more load per position (600 x 2^18 compensated: 4 CTAs 101 us, 5 107, 6
+// 125); scalar loads need the most threads (20011 x 8195 int64: 8 CTAs 98 us, 6
+// 100, 5 106), compensated 128-bit loads run at HBM's rate with 5
+template <class Op, int V, bool DOT>
+constexpr int flat_blocks() { return DOT ? 4 : V == 4 && sizeof(typename Op::Acc) == 8 ? 5 : 8; }
+
+template <class Op, int V, bool DOT>
+__global__ void __launch_bounds__(kFlatThreads, (flat_blocks<Op, V, DOT>()))
+    rect_flat_kernel(const FlatArgs g, const typename Op::In* __restrict__ A, const typename Op::In* __restrict__ w,
+                     typename Op::Out* out, typename Op::Acc* part, float* comp) {
+  using Acc = typename Op::Acc;
+  using In = typename Op::In;
+  constexpr int NL = V == 4 ? 4 : 8;           // loads in flight before the first fold
+  __shared__ Acc wpart[2][kFlatThreads / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int s0 = warp * g.cw + (lane / g.grp_lanes) * g.cg + (lane % g.grp_lanes) * g.cl;
+  const int P = g.P;
+  int buf = 0;
+  for (int64_t item = blockIdx.x; item < g.items; item += gridDim.x, buf ^= 1) {
+    int64_t o = item, lo = 0, n64 = g.R;
+    if (g.G > 1) {
+      o = item / g.G;
+      lo = (item - o * g.G) * g.tile;
+      n64 = g.R - lo < g.tile ? g.R - lo : g.tile;
+    }
+    const int n = static_cast<int>(n64);
+    const In* a = A + o * g.R + lo;
+    const In* wp = DOT ? w + lo : nullptr;
+    Acc acc[1][V];
+#pragma unroll
+    for (int i = 0; i < V; ++i) acc[0][i] = Op::ident();
+    int x = s0;
+    for (; x < n - (NL - 1) * P; x += NL * P) {
+      Vals<Op, V> v[NL][1];
+      In b[NL][V];
+#pragma unroll
+      for (int q = 0; q < NL; ++q) {
+        load_row<In, V>(a + x + q * P, v[q][0].a);
+        if constexpr (DOT) load_bcast<In, V>(wp + x + q * P, b[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < NL; ++q) fold_rows<Op, V, DOT, 1>(acc, v[q], b[q]);
+    }
+    for (; x < n; x += P) {
+      Vals<Op, V> v[1];
+      In b[V];
+      load_row<In, V>(a + x, v[0].a);
+      if constexpr (DOT) load_bcast<In, V>(wp + x, b);
+      fold_rows<Op, V, DOT, 1>(acc, v, b);
+    }
+    const Acc r = lanes_allreduce<Op>(fold_vec<Op, V>(acc[0]), 32);
+    if (lane == 0) wpart[buf][warp] = r;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      Acc t = wpart[buf][0];
+      for (int q = 1; q < g.W; ++q) t = Op::combine(t, wpart[buf][q]);
+      if (g.G > 1) {
+        part[item] = t;
+      } else {
+        out[o] = Op::finish(t);
+        if constexpr (std::is_same_v<Acc, f2>) {
+          if (comp) comp[o] = Op::residual(t);
+        }
+      }
+    }
+  }
+}
+
 // Teams of one lane (rows of 5 to 32 elements) or two (odd rows of up to 64): the
 // rows of a warp's teams are one contiguous block, so the warp copies it to
 // shared memory with 16-byte cp.async (its stage ring keeps the next two blocks
@@ -837,44 +922,17 @@ __global__ void __launch_bounds__(kRowsThreads) rect_thread_rows_kernel(int64_t 
 }
 
 // ---------------------------------------------------------------- grid parts -> outputs
-// A warp per output: the lanes stage up to 256 parts at a time in shared
-// memory with coalesced loads, and lane 0 folds them in part order (the steps
-// of combine_parts, so the bits equal the batched executors').  256 threads.
+// A warp per output, a chain of parts per lane (combine_parts_warp).
 constexpr int kCombineWarps = 8;
-constexpr int kCombineChunk = 256;
 template <class Op>
 __global__ void __launch_bounds__(32 * kCombineWarps) rect_combine_kernel(int64_t O, int32_t G,
                                                                         const typename Op::Acc* part,
                                                                         typename Op::Out* out, float* comp) {
-  using Acc = typename Op::Acc;
-  __shared__ Acc stage[kCombineWarps][kCombineChunk];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int64_t o = blockIdx.x * static_cast<int64_t>(kCombineWarps) + warp; o < O;
        o += static_cast<int64_t>(gridDim.x) * kCombineWarps) {
-    const Acc* pp = part + o * G;
-    PartFold<Op> f;
-    for (int32_t c0 = 0; c0 < G; c0 += kCombineChunk) {
-      const int n = G - c0 < kCombineChunk ? G - c0 : kCombineChunk;
-      for (int i = lane; i < n; i += 32) stage[warp][i] = pp[c0 + i];
-      __syncwarp();
-      if (lane == 0) {
-        int i = 0;
-        if (c0 == 0) {
-          f.first(stage[warp][0]);
-          i = 1;
-        }
-        for (; i + 8 <= n; i += 8) {   // eight shared-memory loads before their folds
-          Acc v[8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) v[k] = stage[warp][i + k];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) f.add(v[k]);
-        }
-        for (; i < n; ++i) f.add(stage[warp][i]);
-      }
-      __syncwarp();
-    }
-    if (lane == 0) out[o] = f.result(comp ? comp + o : nullptr);
+    const typename Op::Out r = combine_parts_warp<Op>(part + o * G, G, lane, comp ? comp + o : nullptr);
+    if (lane == 0) out[o] = r;
   }
 }
 

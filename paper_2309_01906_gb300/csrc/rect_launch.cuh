@@ -83,6 +83,49 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
   return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_rows_kernel launch");
 }
 
+// Does an item of this block-team plan lie in consecutive elements that
+// rect_flat_kernel can fold?
+inline bool flat_plan(const RectPlan& rp) {
+  return rp.team == TEAM_BLOCK && rp.C == 1 && rp.W <= kFlatThreads / 32 && rp.nv == 1 && rp.vstride[0] == 1 &&
+         !rp.pipe && rp.R >= 1 && (rp.G > 1 ? rp.split && rp.tile < (int64_t(1) << 30) : rp.R < (int64_t(1) << 30));
+}
+
+// the second pass over grid parts
+template <class Op>
+hp_status launch_combine(const RectPlan& rp, int sms, const RectArgs& a) {
+  const int64_t cb = (rp.O + kCombineWarps - 1) / kCombineWarps;   // a warp per output
+  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(cb, 4LL * sms));
+  rect_combine_kernel<Op><<<static_cast<int>(grid), 32 * kCombineWarps, 0, a.stream>>>(
+      rp.O, rp.G, static_cast<const typename Op::Acc*>(a.part), static_cast<typename Op::Out*>(a.out), a.comp);
+  const cudaError_t e = cudaPeekAtLastError();
+  return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_combine_kernel launch");
+}
+
+template <class Op, int V, bool DOT>
+hp_status launch_flat(const RectPlan& rp, LaunchCfg& cfg, const typename Op::In* A, const typename Op::In* w,
+                      const RectArgs& a) {
+  auto k = rect_flat_kernel<Op, V, DOT>;
+  if (!cfg.ready) {
+    cfg.threads = 32 * rp.W;
+    int per_sm = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, cfg.threads, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    if (per_sm < 1) return fail(HP_EUNSUPPORTED, "kernel does not fit on an SM with this CTA size");
+    // as many CTAs as run in whole rounds of the items
+    const int64_t resident = static_cast<int64_t>(per_sm) * cfg.sms;
+    const int64_t rounds = std::max<int64_t>(1, (rp.items + resident - 1) / resident);
+    cfg.grid = static_cast<int>(std::max<int64_t>(1, rounds > 4 ? resident : (rp.items + rounds - 1) / rounds));
+    cfg.ready = true;
+  }
+  if (rp.items == 0) return HP_OK;
+  const FlatArgs g{rp.items, rp.R, rp.tile, rp.G, rp.vP[0], rp.W, rp.grp_lanes, rp.cw[0], rp.cg[0], rp.cl[0]};
+  k<<<cfg.grid, cfg.threads, 0, a.stream>>>(g, A, w, static_cast<typename Op::Out*>(a.out),
+                                            static_cast<typename Op::Acc*>(a.part), a.comp);
+  const cudaError_t e = cudaPeekAtLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "rect_flat_kernel launch");
+  return rp.G > 1 ? launch_combine<Op>(rp, cfg.sms, a) : HP_OK;
+}
+
 template <class Op, int V, class Body>
 hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Body& body, const RectArgs& a) {
   using Out = typename Op::Out;
@@ -105,6 +148,7 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
   if constexpr (Body::kPipeable) {
     const RowsKind kind = rows_kind(rp, body.A);
     if (kind != ROWS_NONE) return launch_rows<Op, V, Body::kDot>(rp, kind, cfg, body.A, body.wptr(), a);
+    if (flat_plan(rp)) return launch_flat<Op, V, Body::kDot>(rp, cfg, body.A, body.wptr(), a);
   }
   const bool block = rp.team == TEAM_BLOCK;
   constexpr bool kPipeable = Body::kPipeable && V == 4;
@@ -174,8 +218,6 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
       if (blocks > max_blocks) blocks = max_blocks;
       cfg.grid = static_cast<int>(blocks < 1 ? 1 : blocks);
     }
-    const int64_t cb = (rp.O + kCombineWarps - 1) / kCombineWarps;   // a warp per output
-    cfg.combine_grid = static_cast<int>(cb < 4LL * cfg.sms ? (cb > 0 ? cb : 1) : 4LL * cfg.sms);
     cfg.ready = true;
   }
   if (rp.items == 0) return HP_OK;
@@ -214,11 +256,7 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
     e = cudaPeekAtLastError();
     if (e != cudaSuccess) return cuda_fail(e, "rect_lanes_kernel launch");
   }
-  if (rp.G > 1) {
-    rect_combine_kernel<Op><<<cfg.combine_grid, 32 * kCombineWarps, 0, a.stream>>>(rp.O, rp.G, part, out, a.comp);
-    e = cudaPeekAtLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "rect_combine_kernel launch");
-  }
+  if (rp.G > 1) return launch_combine<Op>(rp, cfg.sms, a);
   (void)np;
   return HP_OK;
 }
