@@ -4,15 +4,16 @@
 // The inner level is ragged, so its binding to hardware is chosen per row
 // (Sec. 3.3: a region compiled for several candidate levels, one picked at run
 // time; Sec. 3.8: sub-warp partitions for short rows).  Each run bins the rows
-// by length into classes and runs one kernel per class:
+// by length into classes, and one persistent kernel takes units of them from a
+// work counter (csr_work_kernel), the longest rows first:
 //   class 0  len <= 4      one thread per row            (SEQ)
 //   class 1  len <= 64     a group of 8 lanes per row     (SUBWARP(8))
 //   class 2  len <= 2048   a warp per row                 (WARP)
 //   class 3  len <= 16384  a CTA of 256 threads per row   (CTA)
 //   class 4  longer        chunks of 16384 entries, a CTA per chunk writing
-//                          its partial to the chunk's slot; a second kernel
-//                          folds each row's partials in chunk order (GRID,
-//                          two-pass; double-float for compensated sums).
+//                          its partial to the chunk's slot; a second pass
+//                          folds each row's partials (GRID, two-pass;
+//                          double-float for compensated sums).
 // Within a class, lane t of a row's team folds entries start + t + k*L (L the
 // team's lanes) into 4 accumulators (k mod 4), then the team combines them in
 // a fixed tree; the tree depends on the row's length only, never on which
@@ -52,12 +53,14 @@ constexpr int kCsrClasses = 5;
 constexpr int64_t kCsrLimit0 = 4, kCsrLimit1 = HP_CSR_LIMIT1, kCsrLimit2 = HP_CSR_LIMIT2, kCsrLimit3 = HP_CSR_LIMIT3;  // class bounds (inclusive)
 constexpr int64_t kCsrChunk = HP_CSR_CHUNK;
 static_assert(kCsrLimit3 >= kCsrChunk, "split rows must be longer than one chunk (bounds the chunk slots)");
-constexpr int kCsrCtaThreads = 256;                       // the chunk kernel's CTA
-#ifndef HP_CSR_ROW_CTA_THREADS
-#define HP_CSR_ROW_CTA_THREADS 256                         // the CTA-per-row kernel's CTA
-#endif
-constexpr int kCsrRowCtaThreads = HP_CSR_ROW_CTA_THREADS;
-constexpr int kCsrBinThreads = 256;
+constexpr int kCsrThreads = 256;                          // every kernel's CTA
+// rows of one unit of work, by class: a chunk, a row, 4 rows per warp, 8 rows
+// per 8-lane team, 8 rows per thread
+constexpr int kCsrUnit0 = 8 * kCsrThreads, kCsrUnit1 = kCsrThreads, kCsrUnit2 = 4 * kCsrThreads / 32;
+// up to this many chunk slots the last CTA of the work kernel folds the long
+// rows' partials; beyond, a kernel of its own does (25,000 rows would take one
+// CTA about 200 us)
+constexpr int64_t kCsrTailChunks = 1024;
 constexpr int kCsrHistSmemMax = 12288;                   // bins counted in shared memory
 #ifndef HP_CSR_GROUPS
 #define HP_CSR_GROUPS 2                                   // 128-bit groups of col / val loaded before their folds
@@ -66,17 +69,21 @@ constexpr int kCsrHistSmemMax = 12288;                   // bins counted in shar
 #define HP_CSR_MIN_BLOCKS 5                               // resident CTAs per SM the wide-team kernels' registers allow (48 registers)
 #endif
 
+// Device counters.  They are zero between runs: the work kernel's last CTA
+// clears them, so that a run needs no clearing launch of its own.
+enum CsrCounter { kCntRows = 0 /* .. 4: rows per class */, kCntChunks = 5, kCntUnit = 6, kCntDone = 7,
+                  kCntSlots = 8 /* chunk slots of the run, for the combine kernel; not cleared */, kCsrCounters = 16 };
+
 struct CsrState {
-  int64_t* counters = nullptr;   // [0..4] rows per class, [5] chunk slots, [6..10] scatter cursors
-  int32_t* rows = nullptr;       // row ids grouped by class
+  int64_t* counters = nullptr;
+  int32_t* rows01 = nullptr;     // row ids: class 0 from the front, class 1 from the back
+  int32_t* rows23 = nullptr;     // class 2 from the front, class 3 from the back
   int32_t* chunk_row = nullptr;  // per chunk slot: row id
   int32_t* chunk_idx = nullptr;  // per chunk slot: chunk index within its row
   int32_t* chunk_cnt = nullptr;  // per chunk slot: chunks of its row
   void* part = nullptr;          // per chunk slot: partial accumulator
   int64_t max_chunks = 0;
-  int grid_rows = 0;             // persistent grid sizes
-  int grid_cta = 0;
-  int grid_row_cta = 0;
+  int grid = 0;                  // CTAs of the persistent kernel
 };
 
 // ---------------------------------------------------------------- planning
@@ -156,59 +163,28 @@ __device__ __forceinline__ int row_class(int64_t len, int fixed) {
 
 __device__ __forceinline__ int64_t n_chunks_of(int64_t len) { return len > 0 ? (len + kCsrChunk - 1) / kCsrChunk : 1; }
 
-__global__ void csr_zero_kernel(int64_t* counters, int n, long long* hist, int64_t n_bins) {
-  const int64_t i0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+__device__ __forceinline__ void zero_hist(long long* hist, int64_t n_bins) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  if (i0 < n) counters[i0] = 0;
-  if (hist)
-    for (int64_t i = i0; i < n_bins; i += stride) hist[i] = 0;
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n_bins; i += stride) hist[i] = 0;
 }
+__global__ void csr_zero_kernel(long long* hist, int64_t n_bins) { zero_hist(hist, n_bins); }
 
-// pass 1: rows per class and chunk slots of long rows (warp ballots, one
-// shared-memory add per warp and class, one global add per block and class)
-__global__ void csr_bin_count_kernel(const int64_t* __restrict__ off, int64_t n_rows, int fixed, int64_t* counters) {
-  __shared__ unsigned long long cnt[kCsrClasses + 1];
-  if (threadIdx.x <= kCsrClasses) cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t tile = blockIdx.x * static_cast<int64_t>(blockDim.x); tile < n_rows; tile += stride) {
-    const int64_t i = tile + threadIdx.x;
-    int c = -1;
-    int64_t len = 0;
-    if (i < n_rows) {
-      len = off[i + 1] - off[i];
-      c = row_class(len, fixed);
-    }
-#pragma unroll
-    for (int k = 0; k < kCsrClasses; ++k) {
-      const unsigned m = __ballot_sync(0xffffffffu, c == k);
-      if (lane == 0 && m) atomicAdd(&cnt[k], static_cast<unsigned long long>(__popc(m)));
-    }
-    if (c == 4) atomicAdd(&cnt[kCsrClasses], static_cast<unsigned long long>(n_chunks_of(len)));
-  }
-  __syncthreads();
-  if (threadIdx.x <= kCsrClasses && cnt[threadIdx.x])
-    atomicAdd(reinterpret_cast<unsigned long long*>(&counters[threadIdx.x]), cnt[threadIdx.x]);
-}
+// where row k of class c sits in the row lists
+__device__ __forceinline__ int64_t list_at(int c, int64_t k, int64_t n_rows) { return (c & 1) ? n_rows - 1 - k : k; }
 
-// pass 2: scatter row ids into their class's range (tile by tile: warp ballots
-// give each row its rank, one global add per block and class reserves the
-// tile's range); reserve chunk slots of long rows
-__global__ void __launch_bounds__(kCsrBinThreads) csr_bin_scatter_kernel(
-    const int64_t* __restrict__ off, int64_t n_rows, int fixed, int64_t* counters, int32_t* rows, int32_t* chunk_row,
-    int32_t* chunk_idx, int32_t* chunk_cnt, int64_t max_chunks, int32_t* err) {
-  constexpr int kWarps = kCsrBinThreads / 32;
+// Binning: row ids into their class's list (tile by tile: warp ballots give
+// each row its rank, one global add per block and class reserves the tile's
+// range) and chunk slots of long rows.  Two classes share a list from its two
+// ends, so no counting pass has to place them.  Also clears the fused histogram.
+__global__ void __launch_bounds__(kCsrThreads) csr_bin_kernel(const int64_t* __restrict__ off, int64_t n_rows, int fixed,
+                                                              int64_t* counters, int32_t* rows01, int32_t* rows23,
+                                                              int32_t* chunk_row, int32_t* chunk_idx,
+                                                              int32_t* chunk_cnt, int64_t max_chunks, int32_t* err,
+                                                              long long* hist, int64_t n_bins) {
+  constexpr int kWarps = kCsrThreads / 32;
   __shared__ int wpos[kWarps][kCsrClasses];
   __shared__ long long bbase[kCsrClasses];
-  // class c occupies rows[start_c .. start_c + count_c); cursors live in counters[6 + c]
-  int64_t start[kCsrClasses];
-  int64_t acc = 0;
-#pragma unroll
-  for (int c = 0; c < kCsrClasses; ++c) {
-    start[c] = acc;
-    acc += counters[c];
-  }
+  if (hist) zero_hist(hist, n_bins);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -236,16 +212,17 @@ __global__ void __launch_bounds__(kCsrBinThreads) csr_bin_scatter_kernel(
         tot += v;
       }
       bbase[threadIdx.x] =
-          tot ? static_cast<long long>(atomicAdd(reinterpret_cast<unsigned long long*>(&counters[6 + threadIdx.x]),
+          tot ? static_cast<long long>(atomicAdd(reinterpret_cast<unsigned long long*>(&counters[kCntRows + threadIdx.x]),
                                                  static_cast<unsigned long long>(tot)))
               : 0;
     }
     __syncthreads();
-    if (c >= 0) rows[start[c] + bbase[c] + wpos[warp][c] + rank] = static_cast<int32_t>(i);
+    if (c >= 0 && c < 4)
+      (c < 2 ? rows01 : rows23)[list_at(c, bbase[c] + wpos[warp][c] + rank, n_rows)] = static_cast<int32_t>(i);
     if (c == 4) {
       const int64_t nc = n_chunks_of(len);
       const unsigned long long base =
-          atomicAdd(reinterpret_cast<unsigned long long*>(&counters[11]), static_cast<unsigned long long>(nc));
+          atomicAdd(reinterpret_cast<unsigned long long*>(&counters[kCntChunks]), static_cast<unsigned long long>(nc));
       if (static_cast<int64_t>(base) + nc > max_chunks) {  // offsets disagree with the declared nnz
         atomicExch(err, 2);
       } else {
@@ -411,56 +388,6 @@ __device__ __forceinline__ void hist_flush(const CsrArgs& a, int* sh) {
     if (sh[i]) atomicAdd(reinterpret_cast<unsigned long long*>(&a.hist[i]), static_cast<unsigned long long>(sh[i]));
 }
 
-// classes 0..2: a team of L lanes (1, 8 or 32) per row; persistent over the class list
-template <class Op, int L, bool HIST>
-__global__ void __launch_bounds__(256, HP_CSR_MIN_BLOCKS) csr_rows_kernel(CsrArgs a, const int32_t* __restrict__ rows, const int64_t* counters,
-                                                       int cls) {
-  extern __shared__ int sh_hist[];
-  if constexpr (HIST) {
-    if (a.smem_bins) hist_init(sh_hist, a.smem_bins);
-  }
-  int64_t start = 0;
-  for (int c = 0; c < cls; ++c) start += counters[c];
-  const int64_t count = counters[cls];
-  const int lane = threadIdx.x & 31;
-  const int lt = lane % L;
-  const int64_t team = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) / L;
-  const int64_t n_teams = static_cast<int64_t>(gridDim.x) * blockDim.x / L;
-  const int64_t warp_first_team = (blockIdx.x * static_cast<int64_t>(blockDim.x) + (threadIdx.x & ~31)) / L;
-  // every lane of a warp runs the same number of rounds (shuffles need the whole warp);
-  // the row id two rounds ahead and the offsets one round ahead are loaded
-  // before the current round's fold, so that their dependent loads overlap it
-  const int64_t dk = team - warp_first_team;
-  int64_t r0 = warp_first_team;
-  int32_t row = r0 + dk < count ? rows[start + r0 + dk] : 0;
-  int32_t row1 = r0 + n_teams + dk < count ? rows[start + r0 + n_teams + dk] : 0;
-  int64_t s0 = r0 + dk < count ? a.off[row] : 0, e0 = r0 + dk < count ? a.off[row + 1] : 0;
-  for (; r0 < count; r0 += n_teams) {
-    const int64_t k = r0 + dk;
-    const bool valid = k < count;
-    const int32_t row2 = k + 2 * n_teams < count ? rows[start + k + 2 * n_teams] : 0;
-    const int64_t s1 = k + n_teams < count ? a.off[row1] : 0;
-    const int64_t e1 = k + n_teams < count ? a.off[row1 + 1] : 0;
-    typename Op::Acc acc[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = Op::ident();
-    if (valid) {
-      if constexpr (L == 32) csr_fold_vec<Op, HIST>(a, sh_hist, s0, e0, lt, L, acc);
-      else csr_fold<Op, HIST>(a, sh_hist, s0, e0, lt, L, acc);
-    }
-    typename Op::Acc r = fold4<Op>(acc);
-    if constexpr (L > 1) r = team_reduce<Op>(r, L);
-    if (valid && lt == 0) a.y[row] = Op::finish(r);
-    row = row1;
-    row1 = row2;
-    s0 = s1;
-    e0 = e1;
-  }
-  if constexpr (HIST) {
-    if (a.smem_bins) hist_flush(a, sh_hist);
-  }
-}
-
 // CTA-wide fold of one entry range; the result is valid in thread 0.  One
 // barrier: callers alternate between the two halves of their warp-partial
 // buffer, so that the next range's partials never overwrite the ones thread 0
@@ -483,74 +410,170 @@ __device__ __forceinline__ typename Op::Acc cta_fold(const CsrArgs& a, int* sh, 
   return r;
 }
 
-// class 3: a CTA per row
-template <class Op, bool HIST>
-__global__ void __launch_bounds__(kCsrRowCtaThreads, HP_CSR_MIN_BLOCKS * kCsrCtaThreads / kCsrRowCtaThreads)
-    csr_cta_kernel(CsrArgs a, const int32_t* __restrict__ rows,
-                                                                 const int64_t* counters) {
-  extern __shared__ int sh_hist[];
-  __shared__ typename Op::Acc wsh[2][kCsrRowCtaThreads / 32];
-  if constexpr (HIST) {
-    if (a.smem_bins) hist_init(sh_hist, a.smem_bins);
-  }
-  int64_t start = 0;
-  for (int c = 0; c < 3; ++c) start += counters[c];
-  const int64_t count = counters[3];
-  int buf = 0;
-  for (int64_t k = blockIdx.x; k < count; k += gridDim.x, buf ^= 1) {
-    const int32_t row = rows[start + k];
-    const typename Op::Acc r = cta_fold<Op, HIST>(a, sh_hist, a.off[row], a.off[row + 1], wsh[buf]);
-    if (threadIdx.x == 0) a.y[row] = Op::finish(r);
-  }
-  if constexpr (HIST) {
-    if (a.smem_bins) hist_flush(a, sh_hist);
-  }
+// a long row's partials (the second pass of Sec. 2's recursive reduction at
+// grid level): the thread of the row's first slot folds them with the grid-part
+// combine (combine_parts), a fixed tree per row
+template <class Op>
+__device__ __forceinline__ void combine_slot(int64_t k, int64_t n_slots, float* y, const int32_t* chunk_row,
+                                             const int32_t* chunk_idx, const int32_t* chunk_cnt,
+                                             const typename Op::Acc* part) {
+  if (chunk_idx[k] != 0) return;
+  const int n = chunk_cnt[k];
+  if (n < 1 || k + n > n_slots) return;   // a row the binning could not place whole (flagged there)
+  y[chunk_row[k]] = combine_parts<Op>(part + k, n, nullptr);
 }
-
-// class 4: a CTA per chunk of a long row; each chunk's partial goes to its
-// slot, and csr_split_combine_kernel folds a row's slots after this kernel
-template <class Op, bool HIST>
-__global__ void __launch_bounds__(kCsrCtaThreads, HP_CSR_MIN_BLOCKS) csr_split_kernel(CsrArgs a, const int64_t* counters,
-                                                                   const int32_t* __restrict__ chunk_row,
-                                                                   const int32_t* __restrict__ chunk_idx,
-                                                                   typename Op::Acc* part, int64_t max_chunks) {
-  extern __shared__ int sh_hist[];
-  __shared__ typename Op::Acc wsh[2][kCsrCtaThreads / 32];
-  if constexpr (HIST) {
-    if (a.smem_bins) hist_init(sh_hist, a.smem_bins);
-  }
-  const int64_t n_slots = counters[11] < max_chunks ? counters[11] : max_chunks;
-  int buf = 0;
-  for (int64_t k = blockIdx.x; k < n_slots; k += gridDim.x, buf ^= 1) {
-    const int32_t row = chunk_row[k];
-    const int64_t c = chunk_idx[k];
-    const int64_t s = a.off[row] + c * kCsrChunk;
-    const int64_t e0 = a.off[row + 1];
-    const int64_t e = (s + kCsrChunk < e0) ? s + kCsrChunk : e0;
-    const typename Op::Acc r = cta_fold<Op, HIST>(a, sh_hist, s, e, wsh[buf]);
-    if (threadIdx.x == 0) part[k] = r;
-  }
-  if constexpr (HIST) {
-    if (a.smem_bins) hist_flush(a, sh_hist);
-  }
-}
-
-// the second pass of long rows (Sec. 2's recursive reduction at grid level):
-// the thread of a row's first slot folds the row's chunk partials in chunk
-// order with the grid-part combine (combine_parts), a fixed tree per row
 template <class Op>
 __global__ void csr_split_combine_kernel(float* __restrict__ y, const int64_t* counters,
                                          const int32_t* __restrict__ chunk_row, const int32_t* __restrict__ chunk_idx,
-                                         const int32_t* __restrict__ chunk_cnt, const typename Op::Acc* __restrict__ part,
-                                         int64_t max_chunks) {
-  const int64_t n_slots = counters[11] < max_chunks ? counters[11] : max_chunks;
+                                         const int32_t* __restrict__ chunk_cnt, const typename Op::Acc* __restrict__ part) {
+  const int64_t n_slots = counters[kCntSlots];
   for (int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; k < n_slots;
-       k += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    if (chunk_idx[k] != 0) continue;
-    const int n = chunk_cnt[k];
-    if (n < 1 || k + n > n_slots) continue;   // a row the binning could not place whole (flagged there)
-    y[chunk_row[k]] = combine_parts<Op>(part + k, n, nullptr);
+       k += static_cast<int64_t>(gridDim.x) * blockDim.x)
+    combine_slot<Op>(k, n_slots, y, chunk_row, chunk_idx, chunk_cnt, part);
+}
+
+struct CsrLists {
+  int64_t* counters;
+  const int32_t* rows01;
+  const int32_t* rows23;
+  const int32_t* chunk_row;
+  const int32_t* chunk_idx;
+  const int32_t* chunk_cnt;
+  int64_t n_rows, max_chunks;
+  int tail_combine;           // 1: the last CTA folds the long rows' partials
+};
+
+// All classes in one persistent kernel: units are taken from a counter, chunks
+// of the longest rows first, single-thread rows last, so one class's waits are
+// filled with another's gathers and only the last units leave SMs idle.  (One
+// kernel per class ran them one after the other, each with its own tail and its
+// own flush of the histogram: 6.37 ms for 4.2 M rows, and nine launches, 61 us,
+// for 300.)  The next unit is claimed before the current one is folded.
+template <class Op, bool HIST>
+__global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kernel(const CsrArgs a, const CsrLists l,
+                                                                                typename Op::Acc* part) {
+  using Acc = typename Op::Acc;
+  extern __shared__ int sh_hist[];
+  __shared__ Acc wsh[2][kCsrThreads / 32];
+  __shared__ uint32_t s_unit, s_first[kCsrClasses], s_rows[3], s_end;
+  __shared__ int s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned long long* const claim = reinterpret_cast<unsigned long long*>(&l.counters[kCntUnit]);
+  if (tid == 0) s_unit = static_cast<uint32_t>(atomicAdd(claim, 1ull));
+  if constexpr (HIST) {
+    if (a.smem_bins) hist_init(sh_hist, a.smem_bins);
   }
+  // the classes' sizes and their first units, longest rows first (fewer than 2^32
+  // units: rows and chunks are below 2^31); in shared memory, to spare registers
+  if (tid == 0) {
+    const int64_t slots = l.counters[kCntChunks] < l.max_chunks ? l.counters[kCntChunks] : l.max_chunks;
+    for (int c = 0; c < 3; ++c) s_rows[c] = static_cast<uint32_t>(l.counters[c]);
+    s_first[4] = 0;
+    s_first[3] = static_cast<uint32_t>(slots);
+    s_first[2] = s_first[3] + static_cast<uint32_t>(l.counters[3]);
+    s_first[1] = s_first[2] + (s_rows[2] + kCsrUnit2 - 1) / kCsrUnit2;
+    s_first[0] = s_first[1] + (s_rows[1] + kCsrUnit1 - 1) / kCsrUnit1;
+    s_end = s_first[0] + (s_rows[0] + kCsrUnit0 - 1) / kCsrUnit0;
+  }
+  __syncthreads();
+  int buf = 0;
+  while (true) {
+    const uint32_t u = s_unit;
+    __syncthreads();   // every thread has read it
+    if (u >= s_end) break;
+    uint32_t next = 0;
+    if (tid == 0) next = static_cast<uint32_t>(atomicAdd(claim, 1ull));
+    if (u < s_first[2]) {      // a chunk of a long row, or a row of the CTA class
+      int64_t s, e;
+      int32_t row;
+      const bool chunk = u < s_first[3];
+      if (chunk) {
+        row = l.chunk_row[u];
+        s = a.off[row] + l.chunk_idx[u] * kCsrChunk;
+        e = a.off[row + 1];
+        if (s + kCsrChunk < e) e = s + kCsrChunk;
+      } else {
+        row = l.rows23[list_at(3, u - s_first[3], l.n_rows)];
+        s = a.off[row];
+        e = a.off[row + 1];
+      }
+      const Acc r = cta_fold<Op, HIST>(a, sh_hist, s, e, wsh[buf]);
+      buf ^= 1;
+      if (tid == 0) {
+        if (chunk) part[u] = r;
+        else a.y[row] = Op::finish(r);
+      }
+    } else if (u < s_first[1]) {   // 4 rows per warp; lane i reads the i-th one's place
+      constexpr int kRows = kCsrUnit2 / (kCsrThreads / 32);
+      const uint32_t k0 = (u - s_first[2]) * kCsrUnit2 + warp * kRows;
+      const int n = k0 >= s_rows[2] ? 0 : static_cast<int>(min(s_rows[2] - k0, static_cast<uint32_t>(kRows)));
+      int32_t id = 0;
+      int64_t s = 0, e = 0;
+      if (lane < n) {
+        id = l.rows23[list_at(2, k0 + lane, l.n_rows)];
+        s = a.off[id];
+        e = a.off[id + 1];
+      }
+      for (int i = 0; i < n; ++i) {
+        Acc acc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = Op::ident();
+        csr_fold_vec<Op, HIST>(a, sh_hist, __shfl_sync(0xffffffffu, s, i), __shfl_sync(0xffffffffu, e, i), lane, 32, acc);
+        const Acc r = team_reduce<Op>(fold4<Op>(acc), 32);
+        if (lane == i) a.y[id] = Op::finish(r);
+      }
+    } else if (u < s_first[0]) {   // 8 lanes per row, 32 rows per warp
+      const uint32_t k0 = (u - s_first[1]) * kCsrUnit1 + warp * 32;
+      int32_t id = -1;
+      int64_t s = 0, e = 0;
+      if (k0 + lane < s_rows[1]) {
+        id = l.rows01[list_at(1, k0 + lane, l.n_rows)];
+        s = a.off[id];
+        e = a.off[id + 1];
+      }
+      for (int i = 0; i < 8; ++i) {
+        const int src = 4 * i + (lane >> 3);
+        const int32_t row = __shfl_sync(0xffffffffu, id, src);
+        const int64_t rs = __shfl_sync(0xffffffffu, s, src), re = __shfl_sync(0xffffffffu, e, src);
+        Acc acc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = Op::ident();
+        if (row >= 0) csr_fold<Op, HIST>(a, sh_hist, rs, re, lane & 7, 8, acc);
+        const Acc r = team_reduce<Op>(fold4<Op>(acc), 8);
+        if (row >= 0 && (lane & 7) == 0) a.y[row] = Op::finish(r);
+      }
+    } else {               // a thread per row
+      const uint32_t k0 = (u - s_first[0]) * kCsrUnit0 + tid;
+      for (int i = 0; i < kCsrUnit0 / kCsrThreads; ++i) {
+        const uint32_t k = k0 + i * kCsrThreads;
+        if (k >= s_rows[0]) break;
+        const int32_t row = l.rows01[list_at(0, k, l.n_rows)];
+        Acc acc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = Op::ident();
+        csr_fold<Op, HIST>(a, sh_hist, a.off[row], a.off[row + 1], 0, 1, acc);
+        a.y[row] = Op::finish(fold4<Op>(acc));
+      }
+    }
+    if (tid == 0) s_unit = next;
+    __syncthreads();
+  }
+  if constexpr (HIST) {
+    if (a.smem_bins) hist_flush(a, sh_hist);
+  }
+  // the last CTA to get here clears the counters for the next run
+  if (tid == 0) {
+    __threadfence();
+    s_last = atomicAdd(reinterpret_cast<unsigned long long*>(&l.counters[kCntDone]), 1ull) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();   // the partials of every CTA are visible
+  if (l.tail_combine)
+    for (int64_t k = tid; k < s_first[3]; k += kCsrThreads)
+      combine_slot<Op>(k, s_first[3], a.y, l.chunk_row, l.chunk_idx, l.chunk_cnt, part);
+  if (tid == 0) l.counters[kCntSlots] = s_first[3];
+  if (tid <= kCntDone) l.counters[tid] = 0;
 }
 
 // standalone count histogram over all entries
@@ -595,35 +618,27 @@ hp_status set_smem(K kernel, size_t dyn) {
 }
 
 template <class Op, bool HIST>
-hp_status launch_classes(hp_nest* n, const CsrArgs& a, cudaStream_t st) {
+hp_status launch_work(hp_nest* n, const CsrArgs& a, cudaStream_t st) {
   CsrState& cs = *n->cs;
   const size_t dyn = HIST ? static_cast<size_t>(a.smem_bins) * sizeof(int) : 0;
-  hp_status s;
-  if ((s = set_smem(csr_rows_kernel<Op, 1, HIST>, dyn)) != HP_OK) return s;
-  if ((s = set_smem(csr_rows_kernel<Op, 8, HIST>, dyn)) != HP_OK) return s;
-  if ((s = set_smem(csr_rows_kernel<Op, 32, HIST>, dyn)) != HP_OK) return s;
-  if ((s = set_smem(csr_cta_kernel<Op, HIST>, dyn)) != HP_OK) return s;
-  if ((s = set_smem(csr_split_kernel<Op, HIST>, dyn)) != HP_OK) return s;
-  const int fixed = n->csr.fixed_class;
-  if (fixed < 0 || fixed == 0) csr_rows_kernel<Op, 1, HIST><<<cs.grid_rows, 256, dyn, st>>>(a, cs.rows, cs.counters, 0);
-  if (fixed < 0 || fixed == 1) csr_rows_kernel<Op, 8, HIST><<<cs.grid_rows, 256, dyn, st>>>(a, cs.rows, cs.counters, 1);
-  if (fixed < 0 || fixed == 2) csr_rows_kernel<Op, 32, HIST><<<cs.grid_rows, 256, dyn, st>>>(a, cs.rows, cs.counters, 2);
-  if (fixed < 0 || fixed == 3)
-    csr_cta_kernel<Op, HIST><<<cs.grid_row_cta, kCsrRowCtaThreads, dyn, st>>>(a, cs.rows, cs.counters);
-  if (fixed < 0 || fixed == 4) {
-    csr_split_kernel<Op, HIST><<<cs.grid_cta, kCsrCtaThreads, dyn, st>>>(
-        a, cs.counters, cs.chunk_row, cs.chunk_idx, static_cast<typename Op::Acc*>(cs.part), cs.max_chunks);
-    const int cgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((cs.max_chunks + 255) / 256, 4 * n->sms)));
-    csr_split_combine_kernel<Op><<<cgrid, 256, 0, st>>>(a.y, cs.counters, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt,
-                                                        static_cast<const typename Op::Acc*>(cs.part), cs.max_chunks);
+  const hp_status s = set_smem(csr_work_kernel<Op, HIST>, dyn);
+  if (s != HP_OK) return s;
+  const bool tail = cs.max_chunks <= kCsrTailChunks;
+  const CsrLists l{cs.counters, cs.rows01, cs.rows23, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt,
+                   n->csr.n_rows, cs.max_chunks, tail ? 1 : 0};
+  typename Op::Acc* part = static_cast<typename Op::Acc*>(cs.part);
+  csr_work_kernel<Op, HIST><<<cs.grid, kCsrThreads, dyn, st>>>(a, l, part);
+  if (!tail) {
+    const int cgrid = static_cast<int>(std::min<int64_t>((cs.max_chunks + 255) / 256, 4 * n->sms));
+    csr_split_combine_kernel<Op><<<cgrid, 256, 0, st>>>(a.y, cs.counters, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, part);
   }
   const cudaError_t e = cudaPeekAtLastError();
-  return e == cudaSuccess ? HP_OK : cuda_fail(e, "CSR class kernel launch");
+  return e == cudaSuccess ? HP_OK : cuda_fail(e, "CSR work kernel launch");
 }
 
 template <class Op>
 hp_status launch_op(hp_nest* n, const CsrArgs& a, cudaStream_t st) {
-  return a.hist ? launch_classes<Op, true>(n, a, st) : launch_classes<Op, false>(n, a, st);
+  return a.hist ? launch_work<Op, true>(n, a, st) : launch_work<Op, false>(n, a, st);
 }
 
 int smem_bins_for(int64_t n_bins) { return n_bins <= kCsrHistSmemMax ? static_cast<int>(n_bins) : 0; }
@@ -637,15 +652,18 @@ hp_status csr_prepare(hp_nest* n) {
   if (!cs) return fail(HP_ENOMEM, "host allocation failed");
   n->cs = cs;
   cudaError_t e;
-  e = cudaMalloc(&cs->counters, 16 * sizeof(int64_t));
+  e = cudaMalloc(&cs->counters, kCsrCounters * sizeof(int64_t));
   if (e != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (CSR counters)");
+  e = cudaMemset(cs->counters, 0, kCsrCounters * sizeof(int64_t));
+  if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (CSR counters)");
   if (p.op == HP_RED_HIST_COUNT) return HP_OK;
   const int64_t rows = std::max<int64_t>(p.n_rows, 1);
   // long rows have > kCsrChunk entries, so chunk slots <= 2 * nnz / kCsrChunk + 1
   cs->max_chunks = 2 * (p.nnz / kCsrChunk) + 2;
   if (p.fixed_class == 4) cs->max_chunks = p.nnz / kCsrChunk + p.n_rows + 2;
-  e = cudaMalloc(&cs->rows, rows * sizeof(int32_t));
-  if (e != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (CSR row lists)");
+  if (cudaMalloc(&cs->rows01, rows * sizeof(int32_t)) != cudaSuccess ||
+      cudaMalloc(&cs->rows23, rows * sizeof(int32_t)) != cudaSuccess)
+    return fail(HP_ENOMEM, "cudaMalloc (CSR row lists)");
   const size_t mc = static_cast<size_t>(cs->max_chunks);
   if (cudaMalloc(&cs->chunk_row, mc * sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&cs->chunk_idx, mc * sizeof(int32_t)) != cudaSuccess ||
@@ -659,17 +677,11 @@ hp_status csr_prepare(hp_nest* n) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (chunk tables)");
   }
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, csr_rows_kernel<OpF32Comp, 32, true>, 256,
-                                                smem_bins_for(p.n_bins) * sizeof(int));
-  cs->grid_rows = std::max(1, per_sm) * n->sms;
-  per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, csr_split_kernel<OpF32Comp, true>, kCsrCtaThreads,
-                                                smem_bins_for(p.n_bins) * sizeof(int));
-  cs->grid_cta = std::max(1, per_sm) * n->sms;
-  per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, csr_cta_kernel<OpF32Comp, true>, kCsrRowCtaThreads,
-                                                smem_bins_for(p.n_bins) * sizeof(int));
-  cs->grid_row_cta = std::max(1, per_sm) * n->sms;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, csr_work_kernel<OpF32Comp, true>, kCsrThreads,
+                                                p.fuse_hist ? smem_bins_for(p.n_bins) * sizeof(int) : 0);
+  // a CTA per 4096 entries and 1024 rows where that is fewer than fit
+  const int64_t want = p.nnz / 4096 + p.n_rows / 1024 + 1;
+  cs->grid = static_cast<int>(std::min<int64_t>(want, static_cast<int64_t>(std::max(1, per_sm)) * n->sms));
   return HP_OK;
 }
 
@@ -684,7 +696,7 @@ hp_status run_csr(hp_nest* n, const void* const* in_dev, void* out_dev, cudaStre
     if (reinterpret_cast<uintptr_t>(col) & 15u) return fail(HP_EINVAL, "col must be 16-byte aligned");
     long long* hist = static_cast<long long*>(out_dev);
     csr_zero_kernel<<<std::max<int64_t>(1, std::min<int64_t>((p.n_bins + 255) / 256, 4 * n->sms)), 256, 0, st>>>(
-        cs.counters, 0, hist, p.n_bins);
+        hist, p.n_bins);
     const int sb = smem_bins_for(p.n_bins);
     const size_t dyn = static_cast<size_t>(sb) * sizeof(int);
     hp_status s = set_smem(csr_hist_kernel, dyn);
@@ -719,15 +731,11 @@ hp_status run_csr(hp_nest* n, const void* const* in_dev, void* out_dev, cudaStre
     a.smem_bins = smem_bins_for(p.n_bins);
   }
   if (p.n_rows == 0) return HP_OK;
-  const int zgrid = static_cast<int>(
-      std::max<int64_t>(1, std::min<int64_t>((std::max<int64_t>(p.fuse_hist ? p.n_bins : 0, 16) + 255) / 256, 4 * n->sms)));
-  csr_zero_kernel<<<zgrid, 256, 0, st>>>(cs.counters, 16, a.hist, p.fuse_hist ? p.n_bins : 0);
-  const int bgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((p.n_rows + kCsrBinThreads - 1) / kCsrBinThreads,
+  const int bgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((p.n_rows + kCsrThreads - 1) / kCsrThreads,
                                                                            8 * n->sms)));
-  csr_bin_count_kernel<<<bgrid, kCsrBinThreads, 0, st>>>(a.off, p.n_rows, p.fixed_class, cs.counters);
-  csr_bin_scatter_kernel<<<bgrid, kCsrBinThreads, 0, st>>>(a.off, p.n_rows, p.fixed_class, cs.counters, cs.rows,
-                                                          cs.chunk_row, cs.chunk_idx, cs.chunk_cnt,
-                                                          cs.max_chunks, n->err);
+  csr_bin_kernel<<<bgrid, kCsrThreads, 0, st>>>(a.off, p.n_rows, p.fixed_class, cs.counters, cs.rows01, cs.rows23,
+                                                cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, cs.max_chunks, n->err, a.hist,
+                                                p.n_bins);
   cudaError_t e = cudaPeekAtLastError();
   if (e != cudaSuccess) return cuda_fail(e, "CSR binning launch");
   switch (p.op) {
@@ -800,7 +808,8 @@ void csr_release(hp_nest* n) {
   CsrState* cs = n->cs;
   if (!cs) return;
   cudaFree(cs->counters);
-  cudaFree(cs->rows);
+  cudaFree(cs->rows01);
+  cudaFree(cs->rows23);
   cudaFree(cs->chunk_row);
   cudaFree(cs->chunk_idx);
   cudaFree(cs->chunk_cnt);
