@@ -177,8 +177,36 @@ struct OrdArgs {
   float* part;        // the state of every (output, part) when G > 1
   int32_t* tickets;   // per output, G > 1
   int64_t O, R, G, part_len, chunk;
+  int64_t total;      // iterations of the whole nest, O * R
   int32_t W;
 };
+
+// Eight consecutive floats at any 4-byte alignment: the three 16-byte granules
+// that hold them, and a shift by the start's place in the first (the same in
+// every lane of a warp, whose pieces are 32 bytes apart).  Scalar loads of a
+// lane's own piece take eight requests for what one 256-bit load brings (33520
+// rows of 1001 maps: 71 us, 50 so).  granules() only loads, so that two arrays'
+// loads overlap; shift() selects.
+struct Granules {
+  float4 a, b, c;
+  uint32_t m;
+  __device__ __forceinline__ void load(const float* __restrict__ x) {
+    m = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(x) >> 2) & 3u;
+    const float4* q = reinterpret_cast<const float4*>(x - m);
+    a = __ldg(q);
+    b = __ldg(q + 1);
+    c = m ? __ldg(q + 2) : b;
+  }
+  __device__ __forceinline__ void shift(float* r) const {
+    float v[11] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) v[k] = (m & 2u) ? v[k + 2] : v[k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) r[k] = (m & 1u) ? v[k + 1] : v[k];
+  }
+};
+// Is every granule of the piece at index i inside an array of n?
+__device__ __forceinline__ bool granules_inside(int64_t i, int64_t n) { return i >= 4 && i + 12 <= n; }
 
 // one 256-bit read-only load (a whole 32-byte sector; the address is 32-byte aligned)
 __device__ __forceinline__ void ld8(const float* p, float* r) {
@@ -189,14 +217,14 @@ __device__ __forceinline__ void ld8(const float* p, float* r) {
 
 // A lane walks its own block, so its loads do not coalesce across the warp:
 // V = 8 takes whole 32-byte sectors with 256-bit loads (each in one request),
-// V = 4 128-bit loads, V = 1 scalar loads.  Every fold runs over [s, e) of the
+// V = 4 128-bit loads, V = 1 shifted granules (whole pieces) and scalar loads.  Every fold runs over [s, e) of the
 // output whose first iteration is `base`, in order.
 
 struct AffineOp {
   using S = float2;   // (A, B)
   static constexpr int kOut = 2;
   template <int V>
-  __device__ static constexpr int64_t piece() { return 8; }   // a lane's iterations per round
+  __host__ __device__ static constexpr int64_t piece() { return 8; }   // a lane's iterations per round
   __device__ static S ident() { return make_float2(1.0f, 0.0f); }
   __device__ static S combine(S e, S l) { return make_float2(__fmul_rn(l.x, e.x), __fmaf_rn(l.x, e.y, l.y)); }
   __device__ static S shfl(S v, int m) {
@@ -213,7 +241,7 @@ struct AffineOp {
 
 template <int V>
 __device__ __forceinline__ float2 fold_affine(const float* __restrict__ a, const float* __restrict__ b, int64_t s,
-                                            int64_t e, float2 v) {
+                                            int64_t e, int64_t total, float2 v) {
   if constexpr (V == 8) {
     for (; s + 16 <= e; s += 16) {
       float av[16], bv[16];
@@ -256,6 +284,24 @@ __device__ __forceinline__ float2 fold_affine(const float* __restrict__ a, const
       v = AffineOp::combine(v, make_float2(a0.w, b0.w));
     }
   } else {
+    for (; s + 8 <= e; s += 8) {
+      float av[8], bv[8];
+      if (granules_inside(s, total)) {
+        Granules ga, gb;
+        ga.load(a + s);
+        gb.load(b + s);
+        ga.shift(av);
+        gb.shift(bv);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          av[q] = __ldg(a + s + q);
+          bv[q] = __ldg(b + s + q);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v = AffineOp::combine(v, make_float2(av[q], bv[q]));
+    }
     for (; s < e; ++s) v = AffineOp::combine(v, make_float2(__ldg(a + s), __ldg(b + s)));
   }
   return v;
@@ -263,14 +309,15 @@ __device__ __forceinline__ float2 fold_affine(const float* __restrict__ a, const
 
 template <int V>
 __device__ __forceinline__ AffineOp::S AffineOp::fold(const OrdArgs& g, int64_t base, int64_t s, int64_t e, S v) {
-  return fold_affine<V>(g.a + base, g.b + base, s, e, v);
+  if constexpr (V == 1) return fold_affine<V>(g.a, g.b, base + s, base + e, g.total, v);
+  else return fold_affine<V>(g.a + base, g.b + base, s, e, g.total, v);
 }
 
 struct Mat2Op {
   using S = float4;   // (m00, m01, m10, m11)
   static constexpr int kOut = 4;
   template <int V>
-  __device__ static constexpr int64_t piece() { return 4; }
+  __host__ __device__ static constexpr int64_t piece() { return 4; }
   __device__ static S ident() { return make_float4(1.0f, 0.0f, 0.0f, 1.0f); }
   __device__ static S combine(S e, S l) {   // L E
     return make_float4(__fmaf_rn(l.x, e.x, __fmul_rn(l.y, e.z)), __fmaf_rn(l.x, e.y, __fmul_rn(l.y, e.w)),
@@ -328,8 +375,10 @@ struct Mat2Op {
 struct LastOp {
   using S = float;    // the last value that is not NaN so far (NaN: none)
   static constexpr int kOut = 1;
+  // shifted granules: the smaller piece keeps a warp's requests to a few lines
+  // each (the result is exact whatever the pieces)
   template <int V>
-  __device__ static constexpr int64_t piece() { return 32; }
+  __host__ __device__ static constexpr int64_t piece() { return V == 1 ? 8 : 32; }
   __device__ static S ident() { return __int_as_float(0x7fc00000); }
   __device__ static S combine(S e, S l) { return l != l ? e : l; }
   __device__ static S shfl(S v, int m) { return __shfl_down_sync(0xffffffffu, v, m); }
@@ -370,6 +419,19 @@ struct LastOp {
         v = combine(combine(combine(combine(v, q.x), q.y), q.z), q.w);
       }
     } else {
+      for (; s + 8 <= e; s += 8) {
+        float r[8];
+        if (granules_inside(base + s, g.total)) {
+          Granules gr;
+          gr.load(a + s);
+          gr.shift(r);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) r[q] = __ldg(a + s + q);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v = combine(v, r[q]);
+      }
       for (; s < e; ++s) v = combine(v, __ldg(a + s));
     }
     return v;
@@ -382,8 +444,7 @@ struct LastOp {
 // lanes combine ranges that are not adjacent); it is the same tree as an xor
 // butterfly's lane 0, with one combine per level and no selects.
 template <class Op>
-__device__ __forceinline__ typename Op::S lanes_in_order(typename Op::S v, int lane) {
-  (void)lane;
+__device__ __forceinline__ typename Op::S lanes_in_order(typename Op::S v) {
 #pragma unroll
   for (int m = 1; m < 32; m <<= 1) v = Op::combine(v, Op::shfl(v, m));
   return v;
@@ -401,7 +462,7 @@ __device__ __forceinline__ typename Op::S fold_warp(const OrdArgs& g, int64_t ba
   for (int64_t r0 = ws; r0 < we; r0 += 32 * P) {
     const int64_t s = std::min<int64_t>(r0 + lane * P, we), e = std::min<int64_t>(s + P, we);
     typename Op::S pc = Op::template fold<V>(g, base, s, e, Op::ident());
-    pc = lanes_in_order<Op>(pc, lane);
+    pc = lanes_in_order<Op>(pc);
     v = Op::combine(v, pc);
   }
   return v;
@@ -414,6 +475,26 @@ __global__ void __launch_bounds__(kOrdThreads) ordered_warp_kernel(OrdArgs g) {
   for (int64_t o = static_cast<int64_t>(blockIdx.x) * (kOrdThreads / 32) + (threadIdx.x >> 5); o < g.O; o += warps) {
     const typename Op::S v = fold_warp<Op, V>(g, o * g.R, 0, g.R, lane);
     if (lane == 0) Op::put(g.out, o, v);
+  }
+}
+
+// Rows of at most 16 pieces: L lanes per output (a power of two, one round of L
+// pieces holds the row), 32 / L outputs per warp.  The tree over L lanes is the
+// whole warp's without the levels that would only join identities.  4.8 M rows of
+// 7 maps: 918 us with a warp each, 51 here.
+template <class Op, int V>
+__global__ void __launch_bounds__(kOrdThreads) ordered_short_kernel(OrdArgs g, int L) {
+  constexpr int64_t P = Op::template piece<V>();
+  const int lane = threadIdx.x & 31, set = 32 / L, lt = lane & (L - 1);
+  const int64_t warps = static_cast<int64_t>(gridDim.x) * (kOrdThreads / 32);
+  const int64_t warp = static_cast<int64_t>(blockIdx.x) * (kOrdThreads / 32) + (threadIdx.x >> 5);
+  for (int64_t first = warp * set; first < g.O; first += warps * set) {   // the same trip count in every lane
+    const int64_t o = first + lane / L;
+    const int64_t s = std::min<int64_t>(lt * P, g.R), e = o < g.O ? std::min<int64_t>(s + P, g.R) : s;
+    typename Op::S v = Op::template fold<V>(g, o * g.R, s, e, Op::ident());
+    for (int m = 1; m < L; m <<= 1) v = Op::combine(v, Op::shfl(v, m));
+    v = Op::combine(Op::ident(), v);   // as the whole warp's round joins its running state
+    if (lt == 0 && o < g.O) Op::put(g.out, o, v);
   }
 }
 
@@ -431,7 +512,7 @@ __global__ void __launch_bounds__(1024) ordered_block_kernel(OrdArgs g) {   // W
     __syncthreads();
     if (warp == 0) {
       typename Op::S w = lane < g.W ? wp[lane] : Op::ident();   // the identity pads the ranks
-      w = lanes_in_order<Op>(w, lane);
+      w = lanes_in_order<Op>(w);
       if (lane == 0) {
         if (g.G == 1) {
           Op::put(g.out, o, w);
@@ -475,10 +556,16 @@ int out_floats(const OrderedPlan& p) {
 template <class Op, int V>
 void launch_ordered(const OrderedPlan& p, const OrdArgs& g, int sms, cudaStream_t st) {
   if (p.team == 0) {
-    auto k = ordered_warp_kernel<Op, V>;
-    const int64_t need = ceil_div(p.O, kOrdThreads / 32);
-    const int grid = static_cast<int>(balanced_grid(need, blocks_for(k, kOrdThreads, sms)));
-    k<<<grid, kOrdThreads, 0, st>>>(g);
+    int L = 32;
+    while (L > 1 && L / 2 * Op::template piece<V>() >= p.R) L /= 2;
+    const int64_t need = ceil_div(p.O, static_cast<int64_t>(kOrdThreads) / L);
+    if (L < 32) {
+      auto k = ordered_short_kernel<Op, V>;
+      k<<<static_cast<int>(balanced_grid(need, blocks_for(k, kOrdThreads, sms))), kOrdThreads, 0, st>>>(g, L);
+    } else {
+      auto k = ordered_warp_kernel<Op, V>;
+      k<<<static_cast<int>(balanced_grid(need, blocks_for(k, kOrdThreads, sms))), kOrdThreads, 0, st>>>(g);
+    }
   } else {
     const int threads = 32 * p.W;
     auto go = [&](auto k) {
@@ -532,6 +619,7 @@ hp_status run_ordered(hp_nest* n, const void* const* in_dev, void* out_dev, cuda
   g.G = p.G;
   g.part_len = std::max<int64_t>(p.part, 1);
   g.chunk = p.chunk;
+  g.total = p.O * p.R;
   g.W = p.W;
   if (reinterpret_cast<uintptr_t>(out_dev) % 4 != 0) return fail(HP_EINVAL, "out must be 4-byte aligned");
   // the widest loads the plan and the input alignment allow (blocks start at whole loads)
