@@ -196,11 +196,18 @@ def _check(st: int, where: str):
         raise HPError(st, where, hp_last_error())
 
 
+# array types of up to 8 pointers, made once: making the type and filling it
+# element by element was half of a call's marshalling
+_PTR_ARRAYS = [ctypes.c_void_p * max(1, n) for n in range(9)]
+
+
 def _ptr_array(ptrs):
-    arr = (ctypes.c_void_p * max(1, len(ptrs)))()
-    for i, v in enumerate(ptrs):
-        arr[i] = ctypes.c_void_p(int(v)) if v else None
-    return arr
+    n = len(ptrs)
+    kind = _PTR_ARRAYS[n] if n < 9 else ctypes.c_void_p * n
+    try:
+        return kind(*ptrs)
+    except TypeError:      # integers of other types (numpy's)
+        return kind(*[int(v) if v else None for v in ptrs])
 
 
 def make_map(levels):
@@ -231,8 +238,9 @@ def hp_nest_create(depth, extents, csr_offsets, n_rows, level_map, op, red_level
 
 
 def hp_nest_run(nest, in_ptrs, out_ptr, stream=0):
-    st = lib().hp_nest_run(nest, _ptr_array(in_ptrs), out_ptr or None, stream or None)
-    _check(st, "hp_nest_run")
+    st = (_lib or lib()).hp_nest_run(nest, _ptr_array(in_ptrs), out_ptr or None, stream or None)
+    if st:
+        _check(st, "hp_nest_run")
 
 
 def hp_nest_run_comp(nest, in_ptrs, out_ptr, comp_ptr, stream=0):
@@ -336,8 +344,9 @@ def hp_serve_create(mem_budget_bytes, max_slots, n_streams):
 
 def hp_serve_submit(server, nest, in_ptrs, out_ptr) -> int:
     t = ctypes.c_uint64()
-    _check(lib().hp_serve_submit(server, nest, _ptr_array(in_ptrs), out_ptr or None, ctypes.byref(t)),
-           "hp_serve_submit")
+    st = (_lib or lib()).hp_serve_submit(server, nest, _ptr_array(in_ptrs), out_ptr or None, ctypes.byref(t))
+    if st:
+        _check(st, "hp_serve_submit")
     return t.value
 
 
@@ -354,7 +363,7 @@ def hp_serve_clock_us() -> float:
 
 def hp_serve_poll(server, ticket, timeout_us=0) -> int:
     """Returns HP_OK (done), HP_EAGAIN (pending) or HP_ETIMEOUT; raises on errors."""
-    st = lib().hp_serve_poll(server, ticket, timeout_us)
+    st = (_lib or lib()).hp_serve_poll(server, ticket, timeout_us)
     if st not in (HP_OK, HP_EAGAIN, HP_ETIMEOUT):
         _check(st, "hp_serve_poll")
     return st
@@ -433,7 +442,9 @@ def hp_stencil_create(ny, nx, radius, coeffs, steps, section=(0, 0), tile=(0, 0)
 
 
 def hp_stencil_run(st, in_ptr, out_ptr, stream=0):
-    _check(lib().hp_stencil_run(st, in_ptr, out_ptr, stream or None), "hp_stencil_run")
+    status = (_lib or lib()).hp_stencil_run(st, in_ptr, out_ptr, stream or None)
+    if status:
+        _check(status, "hp_stencil_run")
 
 
 def hp_stencil_describe(st) -> dict:
