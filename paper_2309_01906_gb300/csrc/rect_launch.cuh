@@ -33,8 +33,9 @@ inline RowsKind rows_kind(const RectPlan& rp, const void* A) {
     return ROWS_NONE;
   // one or two lanes a row: blocks of 32 rows are copied 16 bytes at a time
   const bool aligned = (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
-  if (rp.R >= kThreadRowsMin && aligned && rp.cl[0] == rp.V &&
-      (rp.L == 1 ? rp.R <= 32 : rp.L == 2 && rp.V == 1 && rp.grp_lanes >= 2 && rp.R <= kThreadRowsMax))
+  if (rp.R >= kThreadRowsMin && aligned &&
+      (rp.L == 1 ? rp.R <= 32   // one lane: every slot coefficient is 0
+                 : rp.L == 2 && rp.V == 1 && rp.cl[0] == 1 && rp.grp_lanes >= 2 && rp.R <= kThreadRowsMax))
     return ROWS_THREAD;
   return rp.L > 1 || rp.R < kThreadRowsMin ? ROWS_TEAM : ROWS_NONE;
 }
