@@ -8,6 +8,9 @@
 // leave the registers, and the columns a lane lacks come from its neighbours by
 // shuffle.  The outer R*T columns of the 128 are the ghost zone: they are
 // computed from values the warp does not have, and only the others are stored.
+// At the array's own edges one float4 is ghost zone enough, since what lies
+// outside is known to be 0 at every step, so the first group starts 4 columns
+// before the array (8000 x 116, radius 3, 8 steps: one group instead of two).
 // Likewise a strip starts R*T rows early.  Points outside the array are 0 at
 // every step.  Each point of each step is the same FP32 FMA chain as in the
 // tiled kernel (row-major over the window, from 0), so the bits are equal.
@@ -73,7 +76,9 @@ __global__ void __launch_bounds__(32 * kStreamWarps, MINB)
   const uint32_t st = static_cast<uint32_t>(task / a.n_xt), xt = static_cast<uint32_t>(task - static_cast<uint64_t>(st) * a.n_xt);
   const uint32_t ny = a.ny, nx = a.nx, S = a.S;
   const uint32_t y0 = st * S;                           // first row of the strip
-  const uint32_t gx0 = xt * XW - HX;                    // column of lane 0 (mod 2^32: negative columns are >= nx)
+  constexpr int EX = T == 1 ? 0 : 4;                    // ghost columns at the array's edge
+  const uint32_t gx0 = xt * XW - EX;                    // column of lane 0 (mod 2^32: negative columns are >= nx)
+  const int c_lo = xt == 0 ? EX : HX, c_hi = xt + 1 == a.n_xt ? kStreamCols : kStreamCols - HX;   // columns stored
   const uint32_t gx = gx0 + 4 * lane;
   const int n_it = static_cast<int>(min(S, ny - y0)) + 2 * H;
   const int64_t pitch = a.nx;
@@ -128,7 +133,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, MINB)
 #pragma unroll
       for (int i = 0; i < 4; ++i) A[s][j][i] = 0.0f;
 
-  const bool store_lane = lane >= HX / 4 && lane < 32 - HX / 4 && gx < nx;
+  const bool store_lane = 4 * lane >= c_lo && 4 * lane < c_hi && gx < nx;
   float* op = a.out + static_cast<int64_t>(y0) * pitch + static_cast<int32_t>(VEC ? gx : gx0 + lane);
   int stage = 0, refill = D - 1;
   bool col_in[4];                                       // a 16-byte group is inside the array or outside
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, MINB)
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const int c = lane + 32 * k;
-            if (c >= HX && c < kStreamCols - HX && gx0 + c < nx) op[32 * k] = rg[D][c];
+            if (c >= c_lo && c < c_hi && gx0 + c < nx) op[32 * k] = rg[D][c];
           }
         }
         op += pitch;

@@ -26,8 +26,9 @@ constexpr bool stream_has(int R, int T) { return R >= 1 && R <= 3 ? T >= 1 && T 
 // CTAs of the kernel that fit on an SM (0 if none; CUDA error in *e)
 int stream_occupancy(int R, int T, bool vec, cudaError_t* e);
 
-// columns stored by one warp
+// columns stored by one warp (more at the array's edges), and column groups of a row
 int stream_columns(int R, int T);
+int64_t stream_groups(int64_t nx, int R, int T);
 
 // rows per strip for an ny x nx array when `ctas` CTAs fit on each of `sms` SMs
 uint32_t stream_strip_rows(int64_t ny, int64_t nx, int R, int T, int ctas, int sms);

@@ -42,3 +42,36 @@ def test_streamed_equals_tiled(r, T):
             assert torch.equal(_run(auto, buf, out_offset, ny * nx), want), (ny, nx, out_offset)
         auto.close()
         tiled.close()
+
+
+@pytest.mark.parametrize("r,T", [(1, 2), (2, 7), (3, 8), (4, 2), (4, 5)])
+def test_column_group_edges(r, T):
+    import torch
+    g = np.random.Generator(np.random.PCG64(1000 * r + T))
+    c = g.uniform(-0.5, 0.5, (2 * r + 1) ** 2).astype(np.float32).tolist()
+    probe = hb.Stencil(64, 64, r, c, T)
+    cols = probe.describe()["warp_columns"]
+    probe.close()
+    # one group more from 121 columns on, and again every `cols`; the inner groups overlap by the ghost columns
+    for nx in (119, 120, 121, 124, 120 + cols, 121 + cols, 123 + cols, 120 + 2 * cols, 122 + 2 * cols):
+        A = g.uniform(-1.0, 1.0, 37 * nx).astype(np.float32)
+        buf = torch.from_numpy(A).cuda()
+        auto, tiled = hb.Stencil(37, nx, r, c, T), hb.Stencil(37, nx, r, c, T, tile=(16, 64))
+        assert auto.describe()["kernel"] == "stencil_stream"
+        want = _run(tiled, buf, 0, 37 * nx)
+        assert torch.equal(_run(auto, buf, 0, 37 * nx), want), nx
+        auto.close()
+        tiled.close()
+
+
+@pytest.mark.parametrize("r,T", [(3, 8), (4, 2)])
+def test_long_array_of_one_tile_width(r, T):
+    import torch
+    g = np.random.Generator(np.random.PCG64(7 * r + T))
+    c = g.uniform(-0.5, 0.5, (2 * r + 1) ** 2).astype(np.float32).tolist()
+    A = torch.from_numpy(g.uniform(-1.0, 1.0, 8000 * 128).astype(np.float32)).cuda()
+    auto, tiled = hb.Stencil(8000, 128, r, c, T), hb.Stencil(8000, 128, r, c, T, tile=(16, 64))
+    assert auto.describe()["kernel"] == "stencil_tile"
+    assert torch.equal(_run(auto, A, 0, 8000 * 128), _run(tiled, A, 0, 8000 * 128))
+    auto.close()
+    tiled.close()
