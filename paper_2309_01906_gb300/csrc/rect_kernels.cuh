@@ -705,6 +705,25 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
 #pragma unroll
         for (int q = 0; q < NX; ++q) fold_rows<Op, V, DOT, U>(acc, v[q], b[q]);
       }
+      // the last NX - 1 positions or fewer, again all in flight (2^26 elements in rows of
+      // 900, f32 and int64: 45 and 50 us one after the other, 42 and 41 so); the
+      // compensated folds lose more to its registers (511: 52 us, 72 so)
+      if constexpr (U == 1 && !std::is_same_v<Acc, f2>) {
+        if (x < R) {
+          Vals<Op, V> v[NX - 1][U];
+          In b[NX - 1][V];
+#pragma unroll
+          for (int q = 0; q < NX - 1; ++q) {
+            const int y = x + q * P < R ? x + q * P : x;
+            if constexpr (DOT) load_bcast<In, V>(w + y, b[q]);
+            load_row<In, V>(a + y, v[q][0].a);
+          }
+#pragma unroll
+          for (int q = 0; q < NX - 1; ++q)
+            if (x + q * P < R) fold_rows<Op, V, DOT, U>(acc, v[q], b[q]);
+          x = R;
+        }
+      }
     }
     for (; x < R; x += P) {
       Vals<Op, V> v[U];
@@ -804,12 +823,20 @@ __global__ void __launch_bounds__(kFlatThreads, (flat_blocks<Op, V, DOT>()))
 #pragma unroll
       for (int q = 0; q < NL; ++q) fold_rows<Op, V, DOT, 1>(acc, v[q], b[q]);
     }
-    for (; x < n; x += P) {
-      Vals<Op, V> v[1];
-      In b[V];
-      load_row<In, V>(a + x, v[0].a);
-      if constexpr (DOT) load_bcast<In, V>(wp + x, b);
-      fold_rows<Op, V, DOT, 1>(acc, v, b);
+    // the last NL - 1 positions or fewer, again all in flight (2^26 elements in rows of
+    // 10001: f32 50 us one after the other, 40 so; compensated dot 81 and 64)
+    if (x < n) {
+      Vals<Op, V> v[NL - 1][1];
+      In b[NL - 1][V];
+#pragma unroll
+      for (int q = 0; q < NL - 1; ++q) {
+        const int y = x + q * P < n ? x + q * P : x;
+        load_row<In, V>(a + y, v[q][0].a);
+        if constexpr (DOT) load_bcast<In, V>(wp + y, b[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < NL - 1; ++q)
+        if (x + q * P < n) fold_rows<Op, V, DOT, 1>(acc, v[q], b[q]);
     }
     const Acc r = lanes_allreduce<Op>(fold_vec<Op, V>(acc[0]), 32);
     if (lane == 0) wpart[buf][warp] = r;

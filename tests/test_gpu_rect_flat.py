@@ -36,3 +36,23 @@ def test_flat_blocks_equal_the_batched_executor(prec, op, body):
         torch.cuda.synchronize()
         n.close()
         assert one[O] == 9 and torch.equal(one, many), (O, R)
+
+
+@pytest.mark.parametrize("prec", ["f32", "f32_comp", "i64"])
+def test_long_rows_leave_the_pipeline(prec):
+    import torch
+    s = torch.cuda.current_stream().cuda_stream
+    # around the first row length that leaves it, and tails of one to three more steps of 1024 elements
+    for O, R in [(700, 4092), (700, 4096), (701, 4100), (333, 5120), (91, 6148), (90, 7164), (90, 8188), (33, 8192)]:
+        g = torch.Generator("cuda").manual_seed(O + R)
+        A = torch.randn(O * R, device="cuda", generator=g) if prec[0] == "f" else \
+            torch.randint(-(1 << 30), 1 << 30, (O * R,), dtype=torch.int32, device="cuda", generator=g)
+        n = hb.Nest([O, R], 1, "sum", prec, "load", level_map=["grid", "cta"])
+        assert n.describe()["pipe"] == 1
+        one = torch.full((O + 1,), 9, dtype=torch.int64 if prec == "i64" else A.dtype, device="cuda")
+        many = torch.full_like(one, 9)
+        n.run([A.data_ptr()], one.data_ptr(), s)
+        hb.hp_nest_run_batch([n.handle], [[A.data_ptr()]], [many.data_ptr()], s)
+        torch.cuda.synchronize()
+        n.close()
+        assert one[O] == 9 and torch.equal(one, many), (O, R)
