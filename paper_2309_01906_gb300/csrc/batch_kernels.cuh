@@ -267,8 +267,12 @@ struct RingFold {
   const In* w;
   template <int V>
   __device__ __forceinline__ Vals<Op, V> load(uint32_t off, const In* wp, int32_t x) const {
+    return load_linear<V>(ring + ((off + 4u * static_cast<uint32_t>(x)) & static_cast<uint32_t>(kRingBytes - 1)), wp, x);
+  }
+  // the values at shared address a, the broadcast operand at wp + x
+  template <int V>
+  __device__ __forceinline__ Vals<Op, V> load_linear(uint32_t a, const In* wp, int32_t x) const {
     Vals<Op, V> v;
-    const uint32_t a = ring + ((off + 4u * static_cast<uint32_t>(x)) & static_cast<uint32_t>(kRingBytes - 1));
     if constexpr (V == 4) {
       lds4(a, v.a);
     } else {
@@ -307,25 +311,31 @@ struct RingFold {
   template <int V>
   __device__ __forceinline__ void run_at(uint32_t off, const In* wp, int32_t x0, int32_t x1, int32_t P,
                                          typename Op::Acc (&acc)[V]) const {
+    if (x0 >= x1) return;
     int32_t x = x0;
-    if constexpr (V == 1) {
-      for (; x + 3 * P < x1; x += 4 * P) {
-        const auto v0 = load<V>(off, wp, x);
-        const auto v1 = load<V>(off, wp, x + P);
-        const auto v2 = load<V>(off, wp, x + 2 * P);
-        const auto v3 = load<V>(off, wp, x + 3 * P);
-        apply<V>(acc, v0);
-        apply<V>(acc, v1);
-        apply<V>(acc, v2);
-        apply<V>(acc, v3);
+    const uint32_t a0 = (off + 4u * static_cast<uint32_t>(x0)) & static_cast<uint32_t>(kRingBytes - 1);
+    if (a0 + 4u * static_cast<uint32_t>(x1 - x0) <= static_cast<uint32_t>(kRingBytes)) {
+      // the range does not wrap around the end of the ring: linear addresses
+      constexpr int NL = V == 1 ? 4 : 2;
+      const uint32_t step = 4u * static_cast<uint32_t>(P);
+      uint32_t pa = ring + a0;
+      for (; x + (NL - 1) * P < x1; x += NL * P, pa += NL * step) {
+        Vals<Op, V> v[NL];
+#pragma unroll
+        for (int q = 0; q < NL; ++q) v[q] = load_linear<V>(pa + q * step, wp, x + q * P);
+#pragma unroll
+        for (int q = 0; q < NL; ++q) apply<V>(acc, v[q]);
       }
-    } else {
-      for (; x + P < x1; x += 2 * P) {
-        const auto v0 = load<V>(off, wp, x);
-        const auto v1 = load<V>(off, wp, x + P);
-        apply<V>(acc, v0);
-        apply<V>(acc, v1);
-      }
+      for (; x < x1; x += P, pa += step) apply<V>(acc, load_linear<V>(pa, wp, x));
+      return;
+    }
+    constexpr int NW = V == 1 ? 4 : 2;
+    for (; x + (NW - 1) * P < x1; x += NW * P) {
+      Vals<Op, V> v[NW];
+#pragma unroll
+      for (int q = 0; q < NW; ++q) v[q] = load<V>(off, wp, x + q * P);
+#pragma unroll
+      for (int q = 0; q < NW; ++q) apply<V>(acc, v[q]);
     }
     for (; x < x1; x += P) apply<V>(acc, load<V>(off, wp, x));
   }
@@ -616,7 +626,7 @@ __device__ __forceinline__ void ring_lanes_items(const RingGeom& gm, const Fold&
       ring_wait(rv, e1, ready);
       const uint32_t off = static_cast<uint32_t>(e0) * 4u + fold.shift;
       const uint32_t dist = 4u * static_cast<uint32_t>(teams * R);   // ring bytes between a team's rounds
-      if (L >= kReduceBatch) {
+      if (L >= kReduceBatch && n > 2 * teams) {
         // kReduceBatch rounds (two pairs), then one batched team reduction
         constexpr int B = kReduceBatch;
         for (int j0 = 0; j0 < n; j0 += B * teams) {   // the same trip count in every lane
@@ -638,20 +648,35 @@ __device__ __forceinline__ void ring_lanes_items(const RingGeom& gm, const Fold&
           if ((lt & (L / B - 1)) == 0 && j < n) outp[b + j] = Op::finish(part[0]);
         }
       } else {
+        // One round or two.  Planned teams give a lane 16 to 32 elements, so a
+        // window rarely holds more: reducing kReduceBatch rounds there combined
+        // three identities for every row (batches of rows of 64 to 512,
+        // compensated: 3.3 to 4.2 TB/s so, 4.3 to 5.2 now)
         for (int j0 = 0; j0 < n; j0 += 2 * teams) {   // the same trip count in every lane
           const int ja = j0 + team, jb = ja + teams;
-          Acc accA[V], accB[V];
-#pragma unroll
-          for (int i = 0; i < V; ++i) accA[i] = accB[i] = Op::ident();
           const uint32_t offA = off + 4u * static_cast<uint32_t>(ja * R);
-          if (jb < n) fold.template run_pair<V>(offA, dist, s0, R, gm.P, accA, accB);
-          else if (ja < n) fold.template run_at<V>(offA, fold.w, s0, R, gm.P, accA);
-          const Acc a = lanes_allreduce<Op>(fold_vec<Op, V>(accA), L);
-          // a thread team (L = 1) has no partner to shuffle with: skip the empty second item
-          const Acc c = (L == 1 && jb >= n) ? Op::ident() : lanes_allreduce<Op>(fold_vec<Op, V>(accB), L);
-          if (lt == 0) {
-            if (ja < n) outp[b + ja] = Op::finish(a);
-            if (jb < n) outp[b + jb] = Op::finish(c);
+          Acc accA[V];
+#pragma unroll
+          for (int i = 0; i < V; ++i) accA[i] = Op::ident();
+          if (j0 + teams < n) {
+            Acc accB[V];
+#pragma unroll
+            for (int i = 0; i < V; ++i) accB[i] = Op::ident();
+            if (jb < n) fold.template run_pair<V>(offA, dist, s0, R, gm.P, accA, accB);
+            else if (ja < n) fold.template run_at<V>(offA, fold.w, s0, R, gm.P, accA);
+            Acc part[2] = {fold_vec<Op, V>(accA), fold_vec<Op, V>(accB)};
+            if (L > 1) {
+              lanes_reduce_many<Op, 2>(part, L, lt);
+              const int j = lt < L / 2 ? ja : jb;
+              if ((lt & (L / 2 - 1)) == 0 && j < n) outp[b + j] = Op::finish(part[0]);
+            } else {
+              if (ja < n) outp[b + ja] = Op::finish(part[0]);
+              if (jb < n) outp[b + jb] = Op::finish(part[1]);
+            }
+          } else {
+            if (ja < n) fold.template run_at<V>(offA, fold.w, s0, R, gm.P, accA);
+            const Acc r = lanes_allreduce<Op>(fold_vec<Op, V>(accA), L);
+            if (lt == 0 && ja < n) outp[b + ja] = Op::finish(r);
           }
         }
       }
