@@ -22,6 +22,30 @@
 
 namespace hp {
 
+// Programmatic dependent launch: a kernel launched with launch_dependent() may
+// start while the kernel before it in the stream still runs, once every CTA of
+// that one has called grid_launch_dependents() (or ended); grid_wait() then waits
+// until it has completed and its writes are visible.  Both do nothing in
+// kernels launched the ordinary way.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.gridDim = dim3(static_cast<unsigned>(grid));
+  lc.blockDim = dim3(static_cast<unsigned>(threads));
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+}
+
 struct f2 {
   float s, c;
 };

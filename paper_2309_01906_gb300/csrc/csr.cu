@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(kCsrThreads) csr_bin_kernel(const int64_t* __r
   constexpr int kWarps = kCsrThreads / 32;
   __shared__ int wpos[kWarps][kCsrClasses];
   __shared__ long long bbase[kCsrClasses];
+  grid_launch_dependents();   // the work kernel clears its shared histogram meanwhile
   if (hist) zero_hist(hist, n_bins);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -459,10 +460,11 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned long long* const claim = reinterpret_cast<unsigned long long*>(&l.counters[kCntUnit]);
-  if (tid == 0) s_unit = static_cast<uint32_t>(atomicAdd(claim, 1ull));
   if constexpr (HIST) {
     if (a.smem_bins) hist_init(sh_hist, a.smem_bins);
   }
+  grid_wait();   // the binning
+  if (tid == 0) s_unit = static_cast<uint32_t>(atomicAdd(claim, 1ull));
   // the classes' sizes and their first units, longest rows first (fewer than 2^32
   // units: rows and chunks are below 2^31); in shared memory, to spare registers
   if (tid == 0) {
@@ -627,7 +629,8 @@ hp_status launch_work(hp_nest* n, const CsrArgs& a, cudaStream_t st) {
   const CsrLists l{cs.counters, cs.rows01, cs.rows23, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt,
                    n->csr.n_rows, cs.max_chunks, tail ? 1 : 0};
   typename Op::Acc* part = static_cast<typename Op::Acc*>(cs.part);
-  csr_work_kernel<Op, HIST><<<cs.grid, kCsrThreads, dyn, st>>>(a, l, part);
+  const cudaError_t w = launch_dependent(csr_work_kernel<Op, HIST>, cs.grid, kCsrThreads, dyn, st, a, l, part);
+  if (w != cudaSuccess) return cuda_fail(w, "CSR work kernel launch");
   if (!tail) {
     const int cgrid = static_cast<int>(std::min<int64_t>((cs.max_chunks + 255) / 256, 4 * n->sms));
     csr_split_combine_kernel<Op><<<cgrid, 256, 0, st>>>(a.y, cs.counters, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, part);

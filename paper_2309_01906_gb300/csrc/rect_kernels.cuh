@@ -794,6 +794,7 @@ __global__ void __launch_bounds__(kFlatThreads, (flat_blocks<Op, V, DOT>()))
   using In = typename Op::In;
   constexpr int NL = V == 4 ? 4 : 8;           // loads in flight before the first fold
   __shared__ Acc wpart[2][kFlatThreads / 32];
+  if (g.G > 1) grid_launch_dependents();       // the combine kernel: 2^20 elements 10.2 us with it after, 8.9 so
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int s0 = warp * g.cw + (lane / g.grp_lanes) * g.cg + (lane % g.grp_lanes) * g.cl;
   const int P = g.P;
@@ -956,6 +957,7 @@ __global__ void __launch_bounds__(32 * kCombineWarps) rect_combine_kernel(int64_
                                                                         const typename Op::Acc* part,
                                                                         typename Op::Out* out, float* comp) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  grid_wait();   // launched while the parts are still being folded
   for (int64_t o = blockIdx.x * static_cast<int64_t>(kCombineWarps) + warp; o < O;
        o += static_cast<int64_t>(gridDim.x) * kCombineWarps) {
     const typename Op::Out r = combine_parts_warp<Op>(part + o * G, G, lane, comp ? comp + o : nullptr);

@@ -101,9 +101,9 @@ template <class Op>
 hp_status launch_combine(const RectPlan& rp, int sms, const RectArgs& a) {
   const int64_t cb = (rp.O + kCombineWarps - 1) / kCombineWarps;   // a warp per output
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(cb, 4LL * sms));
-  rect_combine_kernel<Op><<<static_cast<int>(grid), 32 * kCombineWarps, 0, a.stream>>>(
-      rp.O, rp.G, static_cast<const typename Op::Acc*>(a.part), static_cast<typename Op::Out*>(a.out), a.comp);
-  const cudaError_t e = cudaPeekAtLastError();
+  const cudaError_t e = launch_dependent(rect_combine_kernel<Op>, static_cast<int>(grid), 32 * kCombineWarps, 0, a.stream,
+                                         rp.O, rp.G, static_cast<const typename Op::Acc*>(a.part),
+                                         static_cast<typename Op::Out*>(a.out), a.comp);
   return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_combine_kernel launch");
 }
 
