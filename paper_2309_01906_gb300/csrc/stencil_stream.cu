@@ -19,7 +19,7 @@ int64_t stream_groups(int64_t nx, int R, int T) {
 // each step.  Fewer than `busy` CTAs of an SM take as long as that many: 24 warps
 // where memory decides (16384^2, radius 1, 4 steps: 18 warps per SM took 524 us,
 // 28 took 454), about one per scheduler where a row step is hundreds of FMAs
-// (266 x 1848, radius 2, 7 steps: 39 us in strips that fill 12 warps, 23 in
+// (266 x 1848, radius 2, 7 steps: 39 us in strips that fill 12 warps, 27 in
 // longer ones that fill 4, 29 tiled); an underfull last wave costs that share of
 // a whole one.  Over 220 drawn sizes and radii this line took 1.13 times less
 // than 24 warps for all.  Longer strips than 288 rows measured slower than their
