@@ -64,12 +64,14 @@ struct StencilPlan {
   // 95 tiled, radius 4, 2 steps 31 against 23), and the widest ghost zones (24
   // points, 80 of 128 columns kept; radius 4 with 4 steps) where the tiles about
   // fill one wave of 152 CTAs (1500 x 738, radius 3, 8 steps: 129 us against 119, a
-  // second wave, 4499 x 459: 201 against 250; 537 x 1004, radius 4, 4 steps: 46 against 41).
+  // second wave, 4499 x 459: 201 against 250; 537 x 1004, radius 4, 4 steps, 136
+  // tiles: 46 against 41, with 120 tiles the same).
   bool streamed(bool vec) const {
     if (r == 1 && T == 1 && vec) return false;
     if (r >= 3 && T > 1 && stream_groups(nx, r, T) > 1 &&
         ((tiles_x == 1 && tiles_y >= 60) ||
-         ((h >= 24 || (r == 4 && T == 4)) && tiles_y * tiles_x >= 100 && tiles_y * tiles_x <= 152)))
+         (tiles_y * tiles_x <= 152 && ((h >= 24 && tiles_y * tiles_x >= 100) ||
+                                       (r == 4 && T == 4 && tiles_y * tiles_x >= 133)))))
       return false;
     return stream;
   }
