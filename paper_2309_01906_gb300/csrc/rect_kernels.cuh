@@ -862,12 +862,25 @@ __global__ void __launch_bounds__(kFlatThreads, (flat_blocks<Op, V, DOT>()))
 // shared memory with 16-byte cp.async (its stage ring keeps the next two blocks
 // in flight) and the teams fold their rows from there.  Read straight from global
 // memory, such a row takes a sector per team and load: 2^26 elements in rows of
-// 31, f32, 135 us so, 51 here.
+// 31, f32, 135 us so, 46 here.  Short rows come several sets to a block (MANY), so
+// that the waits and the ring's bookkeeping are shared: 2^25 elements in rows of 5,
+// f32 and compensated dot 50 and 62 us with one set, 37 and 52 with up to 736
+// elements, 41 and 54 with 512, 44 and 58 with 1024.  A kernel of its own, since
+// the loop over sets costs longer rows a tenth.  Rows of 4 as whole vectors come
+// here for dot products on two-word accumulators only, whose four rows a thread
+// take too many registers in rect_rows_kernel (compensated 64 us there, 48 here;
+// f32 29 and 33).
 constexpr int kThreadRowsMin = 5, kThreadRowsMax = 64;
 constexpr int kThreadRowsStages = 3;
+constexpr int kThreadRowsElems = 736;
+// sets of rows in a block: at least 16 warps' blocks for every SM
+inline int thread_rows_sets(int64_t O, int64_t R, int L, int sms) {
+  const int64_t set = 32 / L;
+  return static_cast<int>(std::max<int64_t>(1, std::min(kThreadRowsElems / (set * R), O / (set * 16 * std::max(sms, 1)))));
+}
 
-template <class Op, int V, bool DOT>
-__global__ void __launch_bounds__(kRowsThreads) rect_thread_rows_kernel(int64_t O, int R, int L,
+template <class Op, int V, bool DOT, bool MANY>
+__global__ void __launch_bounds__(kRowsThreads) rect_thread_rows_kernel(int64_t O, int R, int L, int K,
                                                                         const typename Op::In* __restrict__ A,
                                                                         const typename Op::In* __restrict__ w,
                                                                         typename Op::Out* out, float* comp) {
@@ -881,15 +894,16 @@ __global__ void __launch_bounds__(kRowsThreads) rect_thread_rows_kernel(int64_t 
     __syncthreads();
   }
   const int set = 32 / L;
-  const int block = set * R;                     // elements of a block; 64 R or 128 R bytes, so blocks keep A's alignment
+  const int rows = MANY ? set * K : set;         // rows of a block: K of every team
+  const int block = rows * R;                    // its elements; whole 64 R or 128 R bytes, so blocks keep A's alignment
   In* const ring = reinterpret_cast<In*>(rows_smem) + warp * kThreadRowsStages * block;
-  const int64_t n_blocks = (O + set - 1) / set;
+  const int64_t n_blocks = (O + rows - 1) / rows;
   const int64_t first = static_cast<int64_t>(blockIdx.x) * (kRowsThreads / 32) + warp;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * (kRowsThreads / 32);
   auto issue = [&](int64_t b, int stage) {
     if (b < n_blocks) {
-      const int64_t left = (O - b * set) * R;    // elements of A from the block on
-      const In* src = A + b * set * R;
+      const int64_t left = (O - b * rows) * R;   // elements of A from the block on
+      const In* src = A + b * rows * R;
       for (int i = 4 * lane; i < block; i += 128) {
         const int n = left - i >= 4 ? 4 : left > i ? static_cast<int>(left - i) : 0;
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(ring + stage * block + i)),
@@ -911,38 +925,42 @@ __global__ void __launch_bounds__(kRowsThreads) rect_thread_rows_kernel(int64_t 
     const In* row = ring + stage * block + lane / L * R;
     refill = stage;
     stage = stage + 1 == kThreadRowsStages ? 0 : stage + 1;
-    Acc acc[1][V];
+    // the same count in every lane
+    for (int j = 0; j < (MANY ? K : 1) && (!MANY || b * rows + j * set < O); ++j, row += set * R) {
+      Acc acc[1][V];
 #pragma unroll
-    for (int i = 0; i < V; ++i) acc[0][i] = Op::ident();
-    for (int x = V * lt; x < R; x += V * L) {
-      Vals<Op, V> v[1];
-      In bb[V];
-      if constexpr (V == 4) {
-        using V4 = typename Vec4Of<In>::T;
-        const V4 q = *reinterpret_cast<const V4*>(row + x);
-        v[0].a[0] = q.x;
-        v[0].a[1] = q.y;
-        v[0].a[2] = q.z;
-        v[0].a[3] = q.w;
-        if constexpr (DOT) {
-          const V4 t = *reinterpret_cast<const V4*>(ws + x);
-          bb[0] = t.x;
-          bb[1] = t.y;
-          bb[2] = t.z;
-          bb[3] = t.w;
+      for (int i = 0; i < V; ++i) acc[0][i] = Op::ident();
+#pragma unroll 4
+      for (int x = V * lt; x < R; x += V * L) {
+        Vals<Op, V> v[1];
+        In bb[V];
+        if constexpr (V == 4) {
+          using V4 = typename Vec4Of<In>::T;
+          const V4 q = *reinterpret_cast<const V4*>(row + x);
+          v[0].a[0] = q.x;
+          v[0].a[1] = q.y;
+          v[0].a[2] = q.z;
+          v[0].a[3] = q.w;
+          if constexpr (DOT) {
+            const V4 t = *reinterpret_cast<const V4*>(ws + x);
+            bb[0] = t.x;
+            bb[1] = t.y;
+            bb[2] = t.z;
+            bb[3] = t.w;
+          }
+        } else {
+          v[0].a[0] = row[x];
+          if constexpr (DOT) bb[0] = ws[x];
         }
-      } else {
-        v[0].a[0] = row[x];
-        if constexpr (DOT) bb[0] = ws[x];
+        fold_rows<Op, V, DOT, 1>(acc, v, bb);
       }
-      fold_rows<Op, V, DOT, 1>(acc, v, bb);
-    }
-    const int64_t o = b * set + lane / L;
-    const Acc t = lanes_allreduce<Op>(fold_vec<Op, V>(acc[0]), L);
-    if (lt == 0 && o < O) {
-      out[o] = Op::finish(t);
-      if constexpr (std::is_same_v<Acc, f2>) {
-        if (comp) comp[o] = Op::residual(t);
+      const int64_t o = b * rows + j * set + lane / L;
+      const Acc t = lanes_allreduce<Op>(fold_vec<Op, V>(acc[0]), L);
+      if (lt == 0 && o < O) {
+        out[o] = Op::finish(t);
+        if constexpr (std::is_same_v<Acc, f2>) {
+          if (comp) comp[o] = Op::residual(t);
+        }
       }
     }
   }

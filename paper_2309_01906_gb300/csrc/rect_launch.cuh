@@ -28,16 +28,21 @@ inline hp_status cuda_fail(cudaError_t e, const char* what) {
 
 // Which kernel folds whole rows (rect_rows_kernel, rect_thread_rows_kernel)?
 enum RowsKind { ROWS_NONE = 0, ROWS_TEAM = 1, ROWS_THREAD = 2 };
-inline RowsKind rows_kind(const RectPlan& rp, const void* A) {
+template <class Op, bool DOT>
+RowsKind rows_kind(const RectPlan& rp, const void* A) {
   if (rp.team != TEAM_LANES || rp.nv != 1 || rp.vstride[0] != 1 || rp.G != 1 || rp.split || rp.R < 1 || rp.R > kRowsMaxR)
     return ROWS_NONE;
   // one or two lanes a row: blocks of 32 rows are copied 16 bytes at a time
   const bool aligned = (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
-  if (rp.R >= kThreadRowsMin && aligned &&
+  constexpr bool kWide = sizeof(typename Op::Acc) == 8, kComp = std::is_same_v<typename Op::Acc, f2>;
+  // vectors of plain rows from 16 elements on load whole sectors anyway (2^25
+  // elements in rows of 16, int64: 27 us in rect_lanes_kernel, 28 through shared memory)
+  const bool sectors = rp.V == 4 && rp.R >= 16 && !DOT && !kComp;
+  if (rp.R >= (kWide && DOT && rp.V == 4 ? 4 : kThreadRowsMin) && aligned && !sectors &&
       (rp.L == 1 ? rp.R <= 32   // one lane: every slot coefficient is 0
                  : rp.L == 2 && rp.V == 1 && rp.cl[0] == 1 && rp.grp_lanes >= 2 && rp.R <= kThreadRowsMax))
     return ROWS_THREAD;
-  return rp.L > 1 || rp.R < kThreadRowsMin ? ROWS_TEAM : ROWS_NONE;
+  return rp.L > 1 || rp.R < 5 ? ROWS_TEAM : ROWS_NONE;
 }
 
 // launch of a rows kernel; cfg is filled on the nest's first run of that kind
@@ -47,9 +52,9 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
   using Out = typename Op::Out;
   auto k1 = rect_rows_kernel<Op, V, DOT, 1>;
   auto k4 = rect_rows_kernel<Op, V, DOT, kRowsU>;
-  auto kt = rect_thread_rows_kernel<Op, V, DOT>;
-  const int set = 32 / rp.L;
-  const size_t dyn = kind == ROWS_THREAD ? sizeof(int32_t) * (kRowsThreads / 32) * kThreadRowsStages * set * rp.R : 0;
+  const int set = 32 / rp.L, K = kind == ROWS_THREAD ? thread_rows_sets(rp.O, rp.R, rp.L, cfg.sms) : 1;
+  auto kt = K > 1 ? rect_thread_rows_kernel<Op, V, DOT, true> : rect_thread_rows_kernel<Op, V, DOT, false>;
+  const size_t dyn = kind == ROWS_THREAD ? sizeof(int32_t) * (kRowsThreads / 32) * kThreadRowsStages * set * K * rp.R : 0;
   const int U = rp.L == 1 ? kRowsU : 1;
   if (!cfg.ready || cfg.rows != kind) {
     const void* f = kind == ROWS_THREAD ? reinterpret_cast<const void*>(kt)
@@ -64,7 +69,7 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kRowsThreads, dyn);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
     if (per_sm < 1) return fail(HP_EUNSUPPORTED, "kernel does not fit on an SM with this CTA size");
-    const int64_t cta_rows = static_cast<int64_t>(kRowsThreads / 32) * set * (kind == ROWS_THREAD ? 1 : U);
+    const int64_t cta_rows = static_cast<int64_t>(kRowsThreads / 32) * set * (kind == ROWS_THREAD ? K : U);
     const int64_t blocks = std::min<int64_t>((rp.O + cta_rows - 1) / cta_rows, static_cast<int64_t>(per_sm) * cfg.sms);
     cfg.threads = kRowsThreads;
     cfg.grid = static_cast<int>(std::max<int64_t>(blocks, 1));
@@ -74,7 +79,7 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
   if (rp.O == 0) return HP_OK;
   Out* out = static_cast<Out*>(a.out);
   if (kind == ROWS_THREAD) {
-    kt<<<cfg.grid, kRowsThreads, dyn, a.stream>>>(rp.O, static_cast<int>(rp.R), rp.L, A, w, out, a.comp);
+    kt<<<cfg.grid, kRowsThreads, dyn, a.stream>>>(rp.O, static_cast<int>(rp.R), rp.L, K, A, w, out, a.comp);
   } else {
     const RowsArgs g{rp.O, static_cast<int32_t>(rp.R), rp.vP[0], rp.L, rp.grp_lanes, rp.cg[0], rp.cl[0]};
     if (U == 1) k1<<<cfg.grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
@@ -152,7 +157,7 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
     return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_map_kernel launch");
   }
   if constexpr (Body::kPipeable) {
-    const RowsKind kind = rows_kind(rp, body.A);
+    const RowsKind kind = rows_kind<Op, Body::kDot>(rp, body.A);
     if (kind != ROWS_NONE) return launch_rows<Op, V, Body::kDot>(rp, kind, cfg, body.A, body.wptr(), a);
     if (flat_plan(rp, Body::kDot)) return launch_flat<Op, V, Body::kDot>(rp, cfg, body.A, body.wptr(), a);
   }

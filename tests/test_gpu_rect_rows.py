@@ -76,3 +76,11 @@ def test_residuals_of_the_rows_kernels():
         # Dot2: the two-word result errs by at most gamma_R^2 sum|t|
         lim = (R * 2.0 ** -24) ** 2 * 4 * A.view(O, R).abs().double().sum(1) + 1e-30
         assert torch.all((out.double() + comp.double() - ref).abs() <= lim)
+
+
+@pytest.mark.parametrize("prec,op,body", [("f32", "sum", "load"), ("f32_comp", "sum", "dot_bcast"), ("i64", "max", "dot_bcast")])
+def test_blocks_of_several_sets(prec, op, body):
+    # enough rows that a warp's block holds several sets of 32; 160001: two, and a ragged last block
+    for R in (4, 5, 7, 8, 11, 15):
+        for O in (160001, 700003):
+            _compare(O, R, op, prec, body, None, 0)
