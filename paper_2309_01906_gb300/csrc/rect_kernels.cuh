@@ -707,8 +707,9 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
       }
       // the last NX - 1 positions or fewer, again all in flight (2^26 elements in rows of
       // 900, f32 and int64: 45 and 50 us one after the other, 42 and 41 so); the
-      // compensated folds lose more to its registers (511: 52 us, 72 so)
-      if constexpr (U == 1 && !std::is_same_v<Acc, f2>) {
+      // compensated folds and dot products lose more to its registers (compensated
+      // 511: 52 us, 72 so; f32 dot of 1200 x 3001: 10 us, 17 so)
+      if constexpr (U == 1 && !DOT && !std::is_same_v<Acc, f2>) {
         if (x < R) {
           Vals<Op, V> v[NX - 1][U];
           In b[NX - 1][V];

@@ -94,10 +94,11 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
 // cp.async pipeline (2^26 elements, f32 / compensated / int64: rows of 4096 44, 54 and
 // 47 us there and 38, 44 and 39 here, 6400 51, 62, 59 and 39, 44, 39, 8192 43, 45, 44
 // and 40, 38, 37); the pipeline stays for dot products (compensated, 7168: 47 there,
-// 53 here), for rows that a round of it holds several of, and for other levels.
-inline bool flat_plan(const RectPlan& rp, bool dot) {
+// 53 here) and 64-bit comparisons (5344: 50 and 52), for rows that a round of it
+// holds several of, and for other levels.
+inline bool flat_plan(const RectPlan& rp, bool leave) {
   return rp.team == TEAM_BLOCK && rp.C == 1 && rp.W <= kFlatThreads / 32 && rp.nv == 1 && rp.vstride[0] == 1 &&
-         (!rp.pipe || (!dot && rp.R >= 4096)) && rp.R >= 1 &&
+         (!rp.pipe || (leave && rp.R >= 4096)) && rp.R >= 1 &&
          (rp.G > 1 ? rp.split && rp.tile < (int64_t(1) << 30) : rp.R < (int64_t(1) << 30));
 }
 
@@ -159,7 +160,8 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
   if constexpr (Body::kPipeable) {
     const RowsKind kind = rows_kind<Op, Body::kDot>(rp, body.A);
     if (kind != ROWS_NONE) return launch_rows<Op, V, Body::kDot>(rp, kind, cfg, body.A, body.wptr(), a);
-    if (flat_plan(rp, Body::kDot)) return launch_flat<Op, V, Body::kDot>(rp, cfg, body.A, body.wptr(), a);
+    constexpr bool kCompare64 = std::is_same_v<Op, OpI64Max> || std::is_same_v<Op, OpI64Min>;
+    if (flat_plan(rp, !Body::kDot && !kCompare64)) return launch_flat<Op, V, Body::kDot>(rp, cfg, body.A, body.wptr(), a);
   }
   const bool block = rp.team == TEAM_BLOCK;
   constexpr bool kPipeable = Body::kPipeable && V == 4;
