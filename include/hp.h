@@ -126,7 +126,8 @@ typedef enum hp_red_op {
  * quiet NaN 0x7fc00000 when there is none (the final value of a forward fill).
  * Exact (error bound 0).  Inputs 32-byte aligned with R (and grid parts) a
  * whole number of 256-bit loads use them; 16-byte aligned, 128-bit loads;
- * otherwise scalar loads, for every ordered operator.
+ * other rows are read as aligned 128-bit loads shifted in registers, for every
+ * ordered operator, and short rows share a warp (the same pieces and tree).
  */
 
 /*
@@ -157,14 +158,15 @@ typedef enum hp_prec {
  * products), in_dev arrays of int8_t / int16_t.  Each thread's 128-bit loads
  * hold 16 (8) elements, 4 sub-lanes (2) in each 32-bit register: sums and
  * dot products accumulate into int32 with __dp4a / __dp2a_lo (exact modulo
- * 2^32), MAX / MIN keep packed running registers (__vmaxs4 / __vmins4,
- * __vmaxs2 / __vmins2) folded over their sub-lanes at the end.  Outputs int32_t
+ * 2^32), MAX / MIN keep packed running registers of 16-bit sub-lanes (an int8
+ * word gives two) folded over their sub-lanes at the end.  Outputs int32_t
  * per output: the sum modulo 2^32, or the max / min value; an empty reduction
  * gives 0 (SUM) or the type's minimum (MAX) / maximum (MIN).  Level map:
  * outputs on GRID, the reduced levels on WARP, CTA (sub_width warps) or GRID
  * (tile > 0: parts combined after a ticket), or AUTO.  Rows whose length or
- * base is not 16-byte aligned take per-element loads (same results).  Not
- * batched, served, tuned or run from host buffers.
+ * base is not 16-byte aligned read 128-bit pieces too, with single loads or
+ * masks for the elements at their ends (same results); short rows share a warp.
+ * Not batched, served, tuned or run from host buffers.
  */
 
 /*
@@ -586,7 +588,9 @@ hp_status hp_nest_tune_req(hp_nest *n, const hp_level_req *req, const void *cons
  * tiles (tile_y x tile_x, tile_x a multiple of 4; 0 = automatic) are mapped
  * into shared memory with a ghost border of r * steps points (one 2-D tensor
  * copy, out-of-array points read as 0), all steps run there, and the CTA
- * writes back its tile.
+ * writes back its tile.  An automatic map without sections may run the streamed
+ * kernel instead (hp_stencil_describe names it): each warp walks a strip of
+ * columns down the rows with every step's values in registers, same results.
  */
 typedef struct hp_stencil hp_stencil;
 typedef struct {

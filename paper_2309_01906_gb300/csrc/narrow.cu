@@ -5,8 +5,8 @@
 // can be split below the lanes.  Here every 32-bit register of a thread's
 // 128-bit load is such a level: sums and int8 dot products go through
 // __dp4a / __dp2a_lo into an int32 accumulator (exact modulo 2^32), maxima and
-// minima through packed running registers (__vmaxs4 / __vmins4, __vmaxs2 /
-// __vmins2) whose sub-lanes are folded once at the end.  Warps combine with
+// minima through packed running registers of two 16-bit lanes (an int8 word is
+// widened to two such) whose sub-lanes are folded once at the end.  Warps combine with
 // the warp-reduce instructions (__reduce_add/max/min_sync), CTAs in shared
 // memory, grid parts after a ticket.  Integer results do not depend on the
 // order, so threads take 16-byte pieces cyclically (coalesced), rows that start
