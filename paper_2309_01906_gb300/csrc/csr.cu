@@ -34,6 +34,7 @@
 
 #include "accum.cuh"
 #include "api_internal.h"
+#include "csr_sequence.h"
 
 namespace hp {
 
@@ -70,7 +71,10 @@ constexpr int kCsrHistSmemMax = 12288;                   // bins counted in shar
 #endif
 
 // Device counters.  They are zero between runs: the work kernel's last CTA
-// clears them, so that a run needs no clearing launch of its own.
+// clears them, so that a run needs no clearing launch of its own (csr_sequence.h
+// has the runs that fail half-way).  Runs of one nest that overlap, which is not
+// allowed, spoil each other's counts; every list position, row id and slot taken
+// from them is bounded all the same and the run is flagged.
 enum CsrCounter { kCntRows = 0 /* .. 4: rows per class */, kCntChunks = 5, kCntUnit = 6, kCntDone = 7,
                   kCntSlots = 8 /* chunk slots of the run, for the combine kernel; not cleared */, kCsrCounters = 16 };
 
@@ -84,6 +88,7 @@ struct CsrState {
   void* part = nullptr;          // per chunk slot: partial accumulator
   int64_t max_chunks = 0;
   int grid = 0;                  // CTAs of the persistent kernel
+  bool dirty = false;            // counters left by a failed run (csr_enqueue)
 };
 
 // ---------------------------------------------------------------- planning
@@ -218,8 +223,11 @@ __global__ void __launch_bounds__(kCsrThreads) csr_bin_kernel(const int64_t* __r
               : 0;
     }
     __syncthreads();
-    if (c >= 0 && c < 4)
-      (c < 2 ? rows01 : rows23)[list_at(c, bbase[c] + wpos[warp][c] + rank, n_rows)] = static_cast<int32_t>(i);
+    if (c >= 0 && c < 4) {
+      const int64_t k = bbase[c] + wpos[warp][c] + rank;
+      if (k < n_rows) (c < 2 ? rows01 : rows23)[list_at(c, k, n_rows)] = static_cast<int32_t>(i);
+      else atomicExch(err, 2);           // counters of another run
+    }
     if (c == 4) {
       const int64_t nc = n_chunks_of(len);
       const unsigned long long base =
@@ -469,10 +477,10 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
   // units: rows and chunks are below 2^31); in shared memory, to spare registers
   if (tid == 0) {
     const int64_t slots = l.counters[kCntChunks] < l.max_chunks ? l.counters[kCntChunks] : l.max_chunks;
-    for (int c = 0; c < 3; ++c) s_rows[c] = static_cast<uint32_t>(l.counters[c]);
+    for (int c = 0; c < 3; ++c) s_rows[c] = static_cast<uint32_t>(min(l.counters[c], l.n_rows));
     s_first[4] = 0;
     s_first[3] = static_cast<uint32_t>(slots);
-    s_first[2] = s_first[3] + static_cast<uint32_t>(l.counters[3]);
+    s_first[2] = s_first[3] + static_cast<uint32_t>(min(l.counters[3], l.n_rows));
     s_first[1] = s_first[2] + (s_rows[2] + kCsrUnit2 - 1) / kCsrUnit2;
     s_first[0] = s_first[1] + (s_rows[1] + kCsrUnit1 - 1) / kCsrUnit1;
     s_end = s_first[0] + (s_rows[0] + kCsrUnit0 - 1) / kCsrUnit0;
@@ -619,29 +627,54 @@ hp_status set_smem(K kernel, size_t dyn) {
   return e == cudaSuccess ? HP_OK : cuda_fail(e, "CSR kernel shared memory");
 }
 
+// one run of a nest with entries (csr_enqueue)
 template <class Op, bool HIST>
-hp_status launch_work(hp_nest* n, const CsrArgs& a, cudaStream_t st) {
-  CsrState& cs = *n->cs;
-  const size_t dyn = HIST ? static_cast<size_t>(a.smem_bins) * sizeof(int) : 0;
-  const hp_status s = set_smem(csr_work_kernel<Op, HIST>, dyn);
-  if (s != HP_OK) return s;
-  const bool tail = cs.max_chunks <= kCsrTailChunks;
-  const CsrLists l{cs.counters, cs.rows01, cs.rows23, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt,
-                   n->csr.n_rows, cs.max_chunks, tail ? 1 : 0};
-  typename Op::Acc* part = static_cast<typename Op::Acc*>(cs.part);
-  const cudaError_t w = launch_dependent(csr_work_kernel<Op, HIST>, cs.grid, kCsrThreads, dyn, st, a, l, part);
-  if (w != cudaSuccess) return cuda_fail(w, "CSR work kernel launch");
-  if (!tail) {
-    const int cgrid = static_cast<int>(std::min<int64_t>((cs.max_chunks + 255) / 256, 4 * n->sms));
-    csr_split_combine_kernel<Op><<<cgrid, 256, 0, st>>>(a.y, cs.counters, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, part);
+struct CsrRun {
+  hp_nest* n;
+  const CsrArgs& a;
+  cudaStream_t st;
+  size_t dyn() const { return HIST ? static_cast<size_t>(a.smem_bins) * sizeof(int) : 0; }
+  hp_status prepare() { return set_smem(csr_work_kernel<Op, HIST>, dyn()); }
+  hp_status clear() {
+    const cudaError_t e = cudaMemsetAsync(n->cs->counters, 0, kCsrCounters * sizeof(int64_t), st);
+    return e == cudaSuccess ? HP_OK : HP_ECUDA;   // the message stays the failed launch's
   }
-  const cudaError_t e = cudaPeekAtLastError();
-  return e == cudaSuccess ? HP_OK : cuda_fail(e, "CSR work kernel launch");
-}
+  hp_status bin() {
+    const CsrPlan& p = n->csr;
+    const CsrState& cs = *n->cs;
+    const int grid = static_cast<int>(
+        std::max<int64_t>(1, std::min<int64_t>((p.n_rows + kCsrThreads - 1) / kCsrThreads, 8 * n->sms)));
+    csr_bin_kernel<<<grid, kCsrThreads, 0, st>>>(a.off, p.n_rows, p.fixed_class, cs.counters, cs.rows01, cs.rows23,
+                                                 cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, cs.max_chunks, n->err, a.hist,
+                                                 p.n_bins);
+    const cudaError_t e = cudaPeekAtLastError();
+    return e == cudaSuccess ? HP_OK : cuda_fail(e, "CSR binning launch");
+  }
+  hp_status work() {
+    const CsrState& cs = *n->cs;
+    const bool tail = cs.max_chunks <= kCsrTailChunks;
+    const CsrLists l{cs.counters, cs.rows01, cs.rows23, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt,
+                     n->csr.n_rows, cs.max_chunks, tail ? 1 : 0};
+    typename Op::Acc* part = static_cast<typename Op::Acc*>(cs.part);
+    const cudaError_t w = launch_dependent(csr_work_kernel<Op, HIST>, cs.grid, kCsrThreads, dyn(), st, a, l, part);
+    if (w != cudaSuccess) return cuda_fail(w, "CSR work kernel launch");
+    if (!tail) {
+      const int cgrid = static_cast<int>(std::min<int64_t>((cs.max_chunks + 255) / 256, 4 * n->sms));
+      csr_split_combine_kernel<Op><<<cgrid, 256, 0, st>>>(a.y, cs.counters, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, part);
+    }
+    const cudaError_t e = cudaPeekAtLastError();
+    return e == cudaSuccess ? HP_OK : cuda_fail(e, "CSR work kernel launch");
+  }
+};
 
 template <class Op>
 hp_status launch_op(hp_nest* n, const CsrArgs& a, cudaStream_t st) {
-  return a.hist ? launch_work<Op, true>(n, a, st) : launch_work<Op, false>(n, a, st);
+  if (a.hist) {
+    CsrRun<Op, true> r{n, a, st};
+    return csr_enqueue(r, &n->cs->dirty, HP_OK);
+  }
+  CsrRun<Op, false> r{n, a, st};
+  return csr_enqueue(r, &n->cs->dirty, HP_OK);
 }
 
 int smem_bins_for(int64_t n_bins) { return n_bins <= kCsrHistSmemMax ? static_cast<int>(n_bins) : 0; }
@@ -673,11 +706,16 @@ hp_status csr_prepare(hp_nest* n) {
       cudaMalloc(&cs->chunk_cnt, mc * sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&cs->part, mc * sizeof(f2)) != cudaSuccess)
     return fail(HP_ENOMEM, "cudaMalloc (CSR chunk tables)");
-  // every slot starts as a valid (row 0, chunk 0) entry, so a slot the binning
-  // could not fill (offsets beyond the declared nnz, flagged) reads in bounds
+  // every slot starts as a valid (row 0, chunk 0) entry and every list place as
+  // row 0, so that one the binning did not fill (offsets beyond the declared
+  // nnz, flagged) reads in bounds
   for (int32_t* t : {cs->chunk_row, cs->chunk_idx, cs->chunk_cnt}) {
     e = cudaMemset(t, 0, mc * sizeof(int32_t));
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (chunk tables)");
+  }
+  for (int32_t* t : {cs->rows01, cs->rows23}) {
+    e = cudaMemset(t, 0, rows * sizeof(int32_t));
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (row lists)");
   }
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, csr_work_kernel<OpF32Comp, true>, kCsrThreads,
@@ -734,13 +772,6 @@ hp_status run_csr(hp_nest* n, const void* const* in_dev, void* out_dev, cudaStre
     a.smem_bins = smem_bins_for(p.n_bins);
   }
   if (p.n_rows == 0) return HP_OK;
-  const int bgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((p.n_rows + kCsrThreads - 1) / kCsrThreads,
-                                                                           8 * n->sms)));
-  csr_bin_kernel<<<bgrid, kCsrThreads, 0, st>>>(a.off, p.n_rows, p.fixed_class, cs.counters, cs.rows01, cs.rows23,
-                                                cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, cs.max_chunks, n->err, a.hist,
-                                                p.n_bins);
-  cudaError_t e = cudaPeekAtLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "CSR binning launch");
   switch (p.op) {
     case HP_RED_SUM:
       return p.prec == HP_F32_COMP ? launch_op<OpF32Comp>(n, a, st) : launch_op<OpF32Sum>(n, a, st);
