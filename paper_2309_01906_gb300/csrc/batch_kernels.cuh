@@ -141,12 +141,13 @@ __device__ __forceinline__ void batch_emit(const EmitTo& to, int64_t item, typen
     part[item] = a;
     __threadfence();  // publish the partial before taking the ticket
     mine = atomicAdd(&to.tickets[o], 1) == to.G - 1;
+    if (mine) __threadfence();  // all parts of this output are visible here
   }
   unsigned last = __ballot_sync(0xffffffffu, mine);
+  if (last) __syncwarp();  // and now to the whole warp (a ballot or a shuffle orders no memory)
   while (last) {
     const int64_t oc = __shfl_sync(0xffffffffu, o, __ffs(last) - 1);
     last &= last - 1;
-    __threadfence();  // all parts of this output are visible
     const typename Op::Out r = combine_parts_warp<Op>(part + oc * to.G, to.G, lane, nullptr);
     if (lane == 0) {
       static_cast<typename Op::Out*>(to.out)[oc] = r;
