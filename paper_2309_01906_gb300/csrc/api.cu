@@ -40,8 +40,9 @@ hp_status ensure_device(hp_nest* n) {
   n->cfg.device = dev;
   e = cudaMalloc(&n->err, sizeof(int32_t));
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (error word)");
-  e = cudaMemset(n->err, 0, sizeof(int32_t));
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (error word)");
+  InitStream init;
+  e = init.zero(n->err, sizeof(int32_t));
+  if (e != cudaSuccess) return cuda_fail(e, "clear error word");
   if (n->kind == NEST_RECT) {
     const RectPlan& rp = n->plan.rp;
     if (rp.G > 1 && rp.items > 0) {
@@ -53,19 +54,21 @@ hp_status ensure_device(hp_nest* n) {
       const size_t b = n->plan.geo_table.size() * sizeof(float);
       e = cudaMalloc(&n->geo, b);
       if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (geometric table)");
-      e = cudaMemcpy(n->geo, n->plan.geo_table.data(), b, cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy (geometric table)");
+      e = init.upload(n->geo, n->plan.geo_table.data(), b);
+      if (e != cudaSuccess) return cuda_fail(e, "upload geometric table");
     }
   } else if (n->kind == NEST_ORDERED) {
-    hp_status st = ordered_prepare(n);
+    hp_status st = ordered_prepare(n, init);
     if (st != HP_OK) return st;
   } else if (n->kind == NEST_NARROW) {
-    hp_status st = narrow_prepare(n);
+    hp_status st = narrow_prepare(n, init);
     if (st != HP_OK) return st;
   } else {
-    hp_status st = csr_prepare(n);
+    hp_status st = csr_prepare(n, init);
     if (st != HP_OK) return st;
   }
+  e = init.wait();
+  if (e != cudaSuccess) return cuda_fail(e, "clear device state");
   n->device = dev;
   return HP_OK;
 }

@@ -6,6 +6,7 @@
 #include <string>
 
 #include "hp_internal.h"
+#include "init_stream.h"
 
 namespace hp {
 enum NestKind : int { NEST_RECT = 0, NEST_CSR = 1, NEST_ORDERED = 2, NEST_NARROW = 3 };
@@ -48,7 +49,7 @@ double error_bound(const hp_nest* n);
 hp_status plan_csr(int depth, int64_t n_rows, const hp_level_map* map, hp_red_op op, int red_level, hp_prec prec,
                    hp_body body, const void* body_params, CsrPlan* out, std::string* why);
 std::string describe_csr(const CsrPlan& p);
-hp_status csr_prepare(hp_nest* n);
+hp_status csr_prepare(hp_nest* n, InitStream& init);
 hp_status run_csr(hp_nest* n, const void* const* in_dev, void* out_dev, cudaStream_t st);
 size_t csr_out_bytes(const hp_nest* n);
 void csr_release(hp_nest* n);
@@ -57,7 +58,7 @@ void csr_release(hp_nest* n);
 hp_status plan_ordered(int depth, const int64_t* extents, const hp_level_map* map, hp_red_op op, int red_level,
                        hp_prec prec, hp_body body, OrderedPlan* out, std::string* why);
 std::string describe_ordered(const OrderedPlan& p);
-hp_status ordered_prepare(hp_nest* n);
+hp_status ordered_prepare(hp_nest* n, InitStream& init);
 hp_status run_ordered(hp_nest* n, const void* const* in_dev, void* out_dev, cudaStream_t st);
 size_t ordered_out_bytes(const OrderedPlan& p);
 
@@ -65,6 +66,6 @@ size_t ordered_out_bytes(const OrderedPlan& p);
 hp_status plan_narrow(int depth, const int64_t* extents, const hp_level_map* map, hp_red_op op, int red_level,
                       hp_prec prec, hp_body body, NarrowPlan* out, std::string* why);
 std::string describe_narrow(const NarrowPlan& p);
-hp_status narrow_prepare(hp_nest* n);
+hp_status narrow_prepare(hp_nest* n, InitStream& init);
 hp_status run_narrow(hp_nest* n, const void* const* in_dev, void* out_dev, cudaStream_t st);
 }  // namespace hp

@@ -160,11 +160,12 @@ hp_status build_ctx(BatchCtx& ctx, hp_nest* const* nests, int count, int dev, in
   for (int b = 0; b < 2; ++b)
     if ((e = cudaMallocHost(&ctx.h_nests[b], sizeof(BatchNest) * std::max(count, 1))) != cudaSuccess)
       return fail(HP_ENOMEM, "cudaMallocHost (batch descriptors)");
-  if (!all.empty() && (e = cudaMemcpy(ctx.d_tiles, all.data(), sizeof(BatchTile) * all.size(),
-                                      cudaMemcpyHostToDevice)) != cudaSuccess)
+  InitStream init;
+  if (!all.empty() && (e = init.upload(ctx.d_tiles, all.data(), sizeof(BatchTile) * all.size())) != cudaSuccess)
     return cuda_err(e, "upload tile table");
-  if ((e = cudaMemset(ctx.d_tickets, 0, sizeof(int32_t) * std::max<int64_t>(tickets, 1))) != cudaSuccess)
+  if ((e = init.zero(ctx.d_tickets, sizeof(int32_t) * std::max<int64_t>(tickets, 1))) != cudaSuccess)
     return cuda_err(e, "zero tickets");
+  if ((e = init.wait()) != cudaSuccess) return cuda_err(e, "batch tables");
   if ((e = cudaStreamCreateWithFlags(&ctx.cap, cudaStreamNonBlocking)) != cudaSuccess)
     return cuda_err(e, "capture stream");
   // the persistent kernels of different arithmetics are independent (own tile

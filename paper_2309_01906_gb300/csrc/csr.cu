@@ -682,7 +682,7 @@ int smem_bins_for(int64_t n_bins) { return n_bins <= kCsrHistSmemMax ? static_ca
 }  // namespace
 
 // ---------------------------------------------------------------- host side
-hp_status csr_prepare(hp_nest* n) {
+hp_status csr_prepare(hp_nest* n, InitStream& init) {
   const CsrPlan& p = n->csr;
   CsrState* cs = new (std::nothrow) CsrState();
   if (!cs) return fail(HP_ENOMEM, "host allocation failed");
@@ -690,8 +690,8 @@ hp_status csr_prepare(hp_nest* n) {
   cudaError_t e;
   e = cudaMalloc(&cs->counters, kCsrCounters * sizeof(int64_t));
   if (e != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (CSR counters)");
-  e = cudaMemset(cs->counters, 0, kCsrCounters * sizeof(int64_t));
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (CSR counters)");
+  e = init.zero(cs->counters, kCsrCounters * sizeof(int64_t));
+  if (e != cudaSuccess) return cuda_fail(e, "clear CSR counters");
   if (p.op == HP_RED_HIST_COUNT) return HP_OK;
   const int64_t rows = std::max<int64_t>(p.n_rows, 1);
   // long rows have > kCsrChunk entries, so chunk slots <= 2 * nnz / kCsrChunk + 1
@@ -710,12 +710,12 @@ hp_status csr_prepare(hp_nest* n) {
   // row 0, so that one the binning did not fill (offsets beyond the declared
   // nnz, flagged) reads in bounds
   for (int32_t* t : {cs->chunk_row, cs->chunk_idx, cs->chunk_cnt}) {
-    e = cudaMemset(t, 0, mc * sizeof(int32_t));
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (chunk tables)");
+    e = init.zero(t, mc * sizeof(int32_t));
+    if (e != cudaSuccess) return cuda_fail(e, "clear chunk tables");
   }
   for (int32_t* t : {cs->rows01, cs->rows23}) {
-    e = cudaMemset(t, 0, rows * sizeof(int32_t));
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (row lists)");
+    e = init.zero(t, rows * sizeof(int32_t));
+    if (e != cudaSuccess) return cuda_fail(e, "clear row lists");
   }
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, csr_work_kernel<OpF32Comp, true>, kCsrThreads,

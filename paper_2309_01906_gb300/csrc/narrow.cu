@@ -560,7 +560,7 @@ cudaError_t launch_narrow_v(const NarrowPlan& p, const NarArgs& g, bool vec, int
 
 }  // namespace
 
-hp_status narrow_prepare(hp_nest* n) {
+hp_status narrow_prepare(hp_nest* n, InitStream& init) {
   const NarrowPlan& p = n->nar;
   if (p.G > 1 && p.O > 0) {
     n->part_bytes = static_cast<size_t>(p.O * p.G) * sizeof(int32_t);
@@ -568,8 +568,8 @@ hp_status narrow_prepare(hp_nest* n) {
     if (e != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (narrow parts)");
     if ((e = cudaMalloc(&n->tickets, sizeof(int32_t) * p.O)) != cudaSuccess)
       return fail(HP_ENOMEM, "cudaMalloc (narrow tickets)");
-    if ((e = cudaMemset(n->tickets, 0, sizeof(int32_t) * p.O)) != cudaSuccess)
-      return fail(HP_ECUDA, std::string("cudaMemset (tickets): ") + cudaGetErrorString(e));
+    if ((e = init.zero(n->tickets, sizeof(int32_t) * p.O)) != cudaSuccess)
+      return fail(HP_ECUDA, std::string("clear tickets: ") + cudaGetErrorString(e));
   }
   return HP_OK;
 }

@@ -587,7 +587,7 @@ void launch_ordered_v(const OrderedPlan& p, const OrdArgs& g, int v, int sms, cu
 
 size_t ordered_out_bytes(const OrderedPlan& p) { return static_cast<size_t>(p.O) * out_floats(p) * sizeof(float); }
 
-hp_status ordered_prepare(hp_nest* n) {
+hp_status ordered_prepare(hp_nest* n, InitStream& init) {
   const OrderedPlan& p = n->ord;
   if (p.G > 1 && p.O > 0) {
     n->part_bytes = static_cast<size_t>(p.O * p.G) * out_floats(p) * sizeof(float);
@@ -595,8 +595,8 @@ hp_status ordered_prepare(hp_nest* n) {
     if (e != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (ordered parts)");
     if ((e = cudaMalloc(&n->tickets, sizeof(int32_t) * p.O)) != cudaSuccess)
       return fail(HP_ENOMEM, "cudaMalloc (ordered tickets)");
-    if ((e = cudaMemset(n->tickets, 0, sizeof(int32_t) * p.O)) != cudaSuccess)
-      return fail(HP_ECUDA, std::string("cudaMemset (tickets): ") + cudaGetErrorString(e));
+    if ((e = init.zero(n->tickets, sizeof(int32_t) * p.O)) != cudaSuccess)
+      return fail(HP_ECUDA, std::string("clear tickets: ") + cudaGetErrorString(e));
   }
   return HP_OK;
 }

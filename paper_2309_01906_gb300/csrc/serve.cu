@@ -406,9 +406,11 @@ hp_status resident_init(hp_server* s) {
       !alloc_mapped(&R.h_ctl, &R.d_ctl, 2) || !alloc_mapped(&R.h_done, &R.d_done, s->max_slots) ||
       !alloc_mapped(&R.h_status, &R.d_status, 2))
     return fail(HP_ENOMEM, "mapped page-locked memory (resident server tables)");
+  InitStream init;
   if (cudaMalloc(&R.d_counts, sizeof(int32_t) * s->max_slots) != cudaSuccess ||
-      cudaMemset(R.d_counts, 0, sizeof(int32_t) * s->max_slots) != cudaSuccess ||
-      cudaMalloc(&R.d_err, sizeof(int32_t)) != cudaSuccess || cudaMemset(R.d_err, 0, sizeof(int32_t)) != cudaSuccess)
+      init.zero(R.d_counts, sizeof(int32_t) * s->max_slots) != cudaSuccess ||
+      cudaMalloc(&R.d_err, sizeof(int32_t)) != cudaSuccess || init.zero(R.d_err, sizeof(int32_t)) != cudaSuccess ||
+      init.wait() != cudaSuccess)
     return fail(HP_ENOMEM, "cudaMalloc (resident tile counts)");
   for (ResidentInst& I : R.inst) {
     if (cudaStreamCreateWithFlags(&I.stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -767,9 +769,10 @@ hp_status hp_serve_create(size_t mem_budget_bytes, int max_slots, int n_streams,
   // scratch pools for grid-split plans: partials and (always zero) tickets
   s->part_cap = std::min<size_t>(mem_budget_bytes / 8 + (1 << 20), size_t(1) << 30);
   s->ticket_cap = std::min<size_t>(mem_budget_bytes / 64 + (1 << 20), size_t(64) << 20);
+  InitStream init;
   if (cudaMalloc(&s->part_pool, s->part_cap) != cudaSuccess ||
       cudaMalloc(reinterpret_cast<void**>(&s->ticket_pool), s->ticket_cap) != cudaSuccess ||
-      cudaMemset(s->ticket_pool, 0, s->ticket_cap) != cudaSuccess) {
+      init.zero(s->ticket_pool, s->ticket_cap) != cudaSuccess || init.wait() != cudaSuccess) {
     hp_serve_destroy(s);
     return fail(HP_ENOMEM, "cudaMalloc (serving scratch pools)");
   }

@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "hp_internal.h"
+#include "init_stream.h"
 #include "stencil_stream.h"
 
 namespace hp {
@@ -478,18 +479,19 @@ hp_status stencil_ensure_device(hp_stencil* s) {
     return stencil_cuda_fail(e, "device query");
   const size_t ob = std::max<size_t>(s->plan.order.size(), 2) * sizeof(int32_t);
   if ((e = cudaMalloc(&s->d_order, ob)) != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (tile order)");
+  InitStream init;
   if (!s->plan.order.empty() &&
-      (e = cudaMemcpy(s->d_order, s->plan.order.data(), s->plan.order.size() * sizeof(int32_t),
-                      cudaMemcpyHostToDevice)) != cudaSuccess)
+      (e = init.upload(s->d_order, s->plan.order.data(), s->plan.order.size() * sizeof(int32_t))) != cudaSuccess)
     return stencil_cuda_fail(e, "upload tile order");
   if ((e = cudaMalloc(&s->err, sizeof(int32_t))) != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (error word)");
-  if ((e = cudaMemset(s->err, 0, sizeof(int32_t))) != cudaSuccess) return stencil_cuda_fail(e, "cudaMemset");
+  if ((e = init.zero(s->err, sizeof(int32_t))) != cudaSuccess) return stencil_cuda_fail(e, "clear error word");
   const StencilPlan& p = s->plan;
   for (int vec = 0; p.stream && vec < 2; ++vec) {
     const int ctas = stream_occupancy(p.r, p.T, vec != 0, &e);
     if (e != cudaSuccess) return stencil_cuda_fail(e, "occupancy query");
     s->strip[vec] = stream_strip_rows(p.ny, p.nx, p.r, p.T, std::max(ctas, 1), s->sms);
   }
+  if ((e = init.wait()) != cudaSuccess) return stencil_cuda_fail(e, "stencil device state");
   s->device = dev;
   return HP_OK;
 }
