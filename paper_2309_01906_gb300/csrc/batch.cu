@@ -17,6 +17,7 @@
 #include <memory>
 #include <mutex>
 #include <numeric>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -37,6 +38,10 @@ struct BatchCtx {
   int32_t* d_tickets = nullptr;
   unsigned long long* d_counters = nullptr;
   std::vector<int64_t> ticket_off;             // per nest (G > 1): offset into d_tickets
+  // a nest listed more than once runs its entries at the same time: those after
+  // the first have partials of their own (else -1: the nest's)
+  unsigned char* d_parts = nullptr;
+  std::vector<int64_t> part_off;
   struct Group {
     int combo;
     int64_t first, n_tiles;
@@ -68,6 +73,7 @@ struct BatchCtx {
     cudaFree(d_nests);
     cudaFree(d_tiles);
     cudaFree(d_tickets);
+    cudaFree(d_parts);
     cudaFree(d_counters);
   }
 };
@@ -110,14 +116,20 @@ void make_tiles(int nest, const RectPlan& rp, int64_t target, std::vector<BatchT
 hp_status build_ctx(BatchCtx& ctx, hp_nest* const* nests, int count, int dev, int sms) {
   ctx.device = dev;
   cudaError_t e;
-  // tickets of grid-split nests
-  int64_t tickets = 0;
+  // tickets of grid-split nests, partials of those listed before
+  int64_t tickets = 0, parts = 0;
   ctx.ticket_off.assign(count, -1);
+  ctx.part_off.assign(count, -1);
+  std::set<const hp_nest*> seen;
   for (int i = 0; i < count; ++i) {
     const RectPlan& rp = nests[i]->plan.rp;
     if (rp.G > 1) {
       ctx.ticket_off[i] = tickets;
       tickets += rp.O;
+      if (!seen.insert(nests[i]).second) {
+        ctx.part_off[i] = parts;
+        parts += static_cast<int64_t>((nests[i]->part_bytes + 15) / 16 * 16);
+      }
     }
   }
   // tile target: about 4 tiles per resident CTA over the whole batch
@@ -155,6 +167,7 @@ hp_status build_ctx(BatchCtx& ctx, hp_nest* const* nests, int count, int dev, in
   if ((e = cudaMalloc(&ctx.d_nests, sizeof(BatchNest) * std::max(count, 1))) != cudaSuccess ||
       (e = cudaMalloc(&ctx.d_tiles, sizeof(BatchTile) * std::max<size_t>(all.size(), 1))) != cudaSuccess ||
       (e = cudaMalloc(&ctx.d_tickets, sizeof(int32_t) * std::max<int64_t>(tickets, 1))) != cudaSuccess ||
+      (parts && (e = cudaMalloc(&ctx.d_parts, static_cast<size_t>(parts))) != cudaSuccess) ||
       (e = cudaMalloc(&ctx.d_counters, sizeof(unsigned long long) * kBatchCombos)) != cudaSuccess)
     return fail(HP_ENOMEM, std::string("cudaMalloc (batch context): ") + cudaGetErrorString(e));
   for (int b = 0; b < 2; ++b)
@@ -292,7 +305,7 @@ extern "C" hp_status hp_nest_run_batch(hp_nest* const* nests, const void* const*
     h[i].in0 = n->plan.n_inputs > 0 ? in_dev[i][0] : nullptr;
     h[i].in1 = n->plan.n_inputs > 1 ? in_dev[i][1] : nullptr;
     h[i].out = out_dev[i];
-    h[i].part = n->part;
+    h[i].part = ctx->part_off[i] >= 0 ? ctx->d_parts + ctx->part_off[i] : n->part;
     h[i].tickets = ctx->ticket_off[i] >= 0 ? ctx->d_tickets + ctx->ticket_off[i] : nullptr;
     h[i].err = n->err;
   }
