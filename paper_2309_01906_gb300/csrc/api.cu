@@ -20,7 +20,7 @@ uint64_t next_plan_id() {
   return ++counter;
 }
 
-hp_status ensure_device(hp_nest* n) {
+hp_status ensure_device(hp_nest* n, const cudaStream_t* run) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e, "no CUDA device");
@@ -40,7 +40,7 @@ hp_status ensure_device(hp_nest* n) {
   n->cfg.device = dev;
   e = cudaMalloc(&n->err, sizeof(int32_t));
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (error word)");
-  InitStream init;
+  InitStream init(run);
   e = init.zero(n->err, sizeof(int32_t));
   if (e != cudaSuccess) return cuda_fail(e, "clear error word");
   if (n->kind == NEST_RECT) {
@@ -54,7 +54,9 @@ hp_status ensure_device(hp_nest* n) {
       const size_t b = n->plan.geo_table.size() * sizeof(float);
       e = cudaMalloc(&n->geo, b);
       if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (geometric table)");
-      e = init.upload(n->geo, n->plan.geo_table.data(), b);
+      InitStream table(nullptr);   // no scratch: such a nest's runs may be unordered
+      e = table.upload(n->geo, n->plan.geo_table.data(), b);
+      if (e == cudaSuccess) e = table.wait();
       if (e != cudaSuccess) return cuda_fail(e, "upload geometric table");
     }
   } else if (n->kind == NEST_ORDERED) {
@@ -235,9 +237,9 @@ hp_status hp_nest_create(int depth, const int64_t* extents, const int64_t* csr_o
 
 hp_status hp_nest_run(hp_nest* n, const void* const* in_dev, void* out_dev, void* stream) {
   if (!n) return fail(HP_EINVAL, "nest is NULL");
-  hp_status st = ensure_device(n);
-  if (st != HP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  hp_status st = ensure_device(n, &s);
+  if (st != HP_OK) return st;
   if (n->kind == NEST_RECT) return run_rect(n, in_dev, out_dev, s);
   if (n->kind == NEST_ORDERED) return run_ordered(n, in_dev, out_dev, s);
   if (n->kind == NEST_NARROW) return run_narrow(n, in_dev, out_dev, s);
@@ -250,19 +252,19 @@ hp_status hp_nest_run_comp(hp_nest* n, const void* const* in_dev, void* out_dev,
     return fail(HP_EUNSUPPORTED, "hp_nest_run_comp takes rectangular compensated FP32 sums (HP_F32_COMP, HP_RED_SUM)");
   const RectPlan& rp = n->plan.rp;
   if (!comp_dev && rp.O > 0) return fail(HP_EINVAL, "comp_dev is NULL");
-  hp_status st = ensure_device(n);
-  if (st != HP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  hp_status st = ensure_device(n, &s);
+  if (st != HP_OK) return st;
   return run_rect_with(n, in_dev, out_dev, n->part, s, static_cast<float*>(comp_dev));
 }
 
 hp_status hp_nest_run_host(hp_nest* n, const void* const* in_host, void* out_host, void* stream) {
   if (!n) return fail(HP_EINVAL, "nest is NULL");
   if (n->kind != NEST_RECT) return fail(HP_EUNSUPPORTED, "hp_nest_run_host takes rectangular nests");
-  hp_status st = ensure_device(n);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  hp_status st = ensure_device(n, &s);
   if (st != HP_OK) return st;
   const NestPlan& p = n->plan;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e;
   const void* dev_in[2] = {nullptr, nullptr};
   for (int i = 0; i < p.n_inputs; ++i) {

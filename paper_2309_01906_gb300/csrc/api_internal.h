@@ -38,7 +38,7 @@ struct hp_nest {
 namespace hp {
 uint64_t next_plan_id();
 void batch_forget(const hp_nest* n);   // drop cached batch contexts that contain n
-hp_status ensure_device(hp_nest* n);
+hp_status ensure_device(hp_nest* n, const cudaStream_t* run);   // run: the first run's stream, nullptr if there is none
 hp_status run_rect(hp_nest* n, const void* const* in_dev, void* out_dev, cudaStream_t st);
 hp_status run_rect_with(hp_nest* n, const void* const* in_dev, void* out_dev, void* part, cudaStream_t st,
                         float* comp = nullptr);

@@ -113,7 +113,7 @@ void make_tiles(int nest, const RectPlan& rp, int64_t target, std::vector<BatchT
   }
 }
 
-hp_status build_ctx(BatchCtx& ctx, hp_nest* const* nests, int count, int dev, int sms) {
+hp_status build_ctx(BatchCtx& ctx, hp_nest* const* nests, int count, int dev, int sms, cudaStream_t run) {
   ctx.device = dev;
   cudaError_t e;
   // tickets of grid-split nests, partials of those listed before
@@ -173,7 +173,7 @@ hp_status build_ctx(BatchCtx& ctx, hp_nest* const* nests, int count, int dev, in
   for (int b = 0; b < 2; ++b)
     if ((e = cudaMallocHost(&ctx.h_nests[b], sizeof(BatchNest) * std::max(count, 1))) != cudaSuccess)
       return fail(HP_ENOMEM, "cudaMallocHost (batch descriptors)");
-  InitStream init;
+  InitStream init(&run);
   if (!all.empty() && (e = init.upload(ctx.d_tiles, all.data(), sizeof(BatchTile) * all.size())) != cudaSuccess)
     return cuda_err(e, "upload tile table");
   if ((e = init.zero(ctx.d_tickets, sizeof(int32_t) * std::max<int64_t>(tickets, 1))) != cudaSuccess)
@@ -253,6 +253,7 @@ extern "C" hp_status hp_nest_run_batch(hp_nest* const* nests, const void* const*
   if (count < 0) return fail(HP_EINVAL, "count must be >= 0");
   if (count == 0) return HP_OK;
   if (!nests || !in_dev || !out_dev) return fail(HP_EINVAL, "NULL argument");
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
   for (int i = 0; i < count; ++i) {
     hp_nest* n = nests[i];
     if (!n) return fail(HP_EINVAL, "nest " + std::to_string(i) + " is NULL");
@@ -260,7 +261,7 @@ extern "C" hp_status hp_nest_run_batch(hp_nest* const* nests, const void* const*
     const NestPlan& p = n->plan;
     const RectPlan& rp = p.rp;
     if (p.body == HP_BODY_GEOMETRIC) return fail(HP_EUNSUPPORTED, "the GEOMETRIC body is not batched");
-    hp_status st = ensure_device(n);
+    hp_status st = ensure_device(n, &s);
     if (st != HP_OK) return st;
     for (int k = 0; k < p.n_inputs; ++k) {
       if (!in_dev[i] || !in_dev[i][k]) return fail(HP_EINVAL, "nest " + std::to_string(i) + ": missing input");
@@ -287,7 +288,7 @@ extern "C" hp_status hp_nest_run_batch(hp_nest* const* nests, const void* const*
     auto c = std::make_unique<BatchCtx>();
     c->key.assign(nests, nests + count);
     for (int i = 0; i < count; ++i) c->ids.push_back(nests[i]->plan_id);
-    hp_status st = build_ctx(*c, nests, count, dev, nests[0]->sms);
+    hp_status st = build_ctx(*c, nests, count, dev, nests[0]->sms, s);
     if (st != HP_OK) return st;
     g_batch_ctx.push_front(std::move(c));
     while (g_batch_ctx.size() > kMaxBatchCtx) g_batch_ctx.pop_back();
@@ -309,7 +310,6 @@ extern "C" hp_status hp_nest_run_batch(hp_nest* const* nests, const void* const*
     h[i].tickets = ctx->ticket_off[i] >= 0 ? ctx->d_tickets + ctx->ticket_off[i] : nullptr;
     h[i].err = n->err;
   }
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   if ((e = cudaGraphLaunch(ctx->exec[b], s)) != cudaSuccess) return cuda_err(e, "batch graph launch");
   // nests the persistent kernel cannot run (cluster teams): their own kernels, same stream
   for (int i = 0; i < count; ++i) {

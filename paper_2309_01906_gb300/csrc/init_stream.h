@@ -5,15 +5,21 @@
 
 namespace hp {
 
-// Clears and fills fresh device memory on a stream of its own; after wait() it is
-// ready for every stream.  cudaMemset, and cudaMemcpy from pageable memory, are
-// queued on the legacy stream and may still be pending when they return, behind
-// whatever the program has queued there, and streams created non-blocking (a
-// user's first run may be on one) do not wait for it.
+// Clears and fills fresh device memory.  cudaMemset, and cudaMemcpy from pageable
+// memory, are queued on the legacy stream and may still be pending when they
+// return, behind whatever the program has queued there, and streams created
+// non-blocking (a user's first run may be on one) do not wait for it.  So the work
+// goes to the stream of the first run, which later runs are ordered after; when
+// there is none, or it is being captured (the work would wait for a replay), to a
+// stream of its own that wait() waits for (a new nest's first run: 96 us on the
+// run's stream, 115 on one of its own).
 class InitStream {
  public:
+  explicit InitStream(const cudaStream_t* run) : run_(run) {}   // the first run's stream, or nullptr
+  InitStream(const InitStream&) = delete;
+  InitStream& operator=(const InitStream&) = delete;
   ~InitStream() {
-    if (s_) cudaStreamDestroy(s_);
+    if (own_) cudaStreamDestroy(s_);
   }
   cudaError_t zero(void* p, size_t bytes) {
     const cudaError_t e = open();
@@ -23,11 +29,27 @@ class InitStream {
     const cudaError_t e = open();
     return e == cudaSuccess ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s_) : e;
   }
-  cudaError_t wait() { return s_ ? cudaStreamSynchronize(s_) : cudaSuccess; }
+  cudaError_t wait() { return own_ ? cudaStreamSynchronize(s_) : cudaSuccess; }
 
  private:
-  cudaError_t open() { return s_ ? cudaSuccess : cudaStreamCreateWithFlags(&s_, cudaStreamNonBlocking); }
+  cudaError_t open() {
+    if (open_) return cudaSuccess;
+    if (run_) {
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(*run_, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        s_ = *run_;
+        open_ = true;
+        return cudaSuccess;
+      }
+      cudaGetLastError();
+    }
+    const cudaError_t e = cudaStreamCreateWithFlags(&s_, cudaStreamNonBlocking);
+    open_ = own_ = e == cudaSuccess;
+    return e;
+  }
+  const cudaStream_t* run_;
   cudaStream_t s_ = nullptr;
+  bool open_ = false, own_ = false;
 };
 
 }  // namespace hp

@@ -406,7 +406,7 @@ hp_status resident_init(hp_server* s) {
       !alloc_mapped(&R.h_ctl, &R.d_ctl, 2) || !alloc_mapped(&R.h_done, &R.d_done, s->max_slots) ||
       !alloc_mapped(&R.h_status, &R.d_status, 2))
     return fail(HP_ENOMEM, "mapped page-locked memory (resident server tables)");
-  InitStream init;
+  InitStream init(nullptr);
   if (cudaMalloc(&R.d_counts, sizeof(int32_t) * s->max_slots) != cudaSuccess ||
       init.zero(R.d_counts, sizeof(int32_t) * s->max_slots) != cudaSuccess ||
       cudaMalloc(&R.d_err, sizeof(int32_t)) != cudaSuccess || init.zero(R.d_err, sizeof(int32_t)) != cudaSuccess ||
@@ -769,7 +769,7 @@ hp_status hp_serve_create(size_t mem_budget_bytes, int max_slots, int n_streams,
   // scratch pools for grid-split plans: partials and (always zero) tickets
   s->part_cap = std::min<size_t>(mem_budget_bytes / 8 + (1 << 20), size_t(1) << 30);
   s->ticket_cap = std::min<size_t>(mem_budget_bytes / 64 + (1 << 20), size_t(64) << 20);
-  InitStream init;
+  InitStream init(nullptr);
   if (cudaMalloc(&s->part_pool, s->part_cap) != cudaSuccess ||
       cudaMalloc(reinterpret_cast<void**>(&s->ticket_pool), s->ticket_cap) != cudaSuccess ||
       init.zero(s->ticket_pool, s->ticket_cap) != cudaSuccess || init.wait() != cudaSuccess) {
@@ -832,7 +832,7 @@ hp_status submit(hp_server* s, const hp_nest* shape, const void* const* in_dev, 
     if (cudaGetDevice(&dev) != cudaSuccess || dev != s->device || (n->device >= 0 && n->device != s->device))
       return fail(HP_EINVAL, "the nest, the calling thread and the server must share one device");
   } else {
-    const hp_status st = ensure_device(n);
+    const hp_status st = ensure_device(n, nullptr);
     if (st != HP_OK) return st;
   }
   for (int i = 0; i < n->plan.n_inputs; ++i)

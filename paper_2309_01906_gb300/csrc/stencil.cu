@@ -479,7 +479,7 @@ hp_status stencil_ensure_device(hp_stencil* s) {
     return stencil_cuda_fail(e, "device query");
   const size_t ob = std::max<size_t>(s->plan.order.size(), 2) * sizeof(int32_t);
   if ((e = cudaMalloc(&s->d_order, ob)) != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (tile order)");
-  InitStream init;
+  InitStream init(nullptr);   // runs of a stencil need not be ordered
   if (!s->plan.order.empty() &&
       (e = init.upload(s->d_order, s->plan.order.data(), s->plan.order.size() * sizeof(int32_t))) != cudaSuccess)
     return stencil_cuda_fail(e, "upload tile order");

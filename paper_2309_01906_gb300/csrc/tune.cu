@@ -168,7 +168,7 @@ hp_status time_runs_graph(hp_nest* tmp, const void* const* in_dev, void* out_dev
 // that microsecond kernels are timed on the device, not by the host's launch
 // rate or the event resolution.
 hp_status time_plan(hp_nest* tmp, const void* const* in_dev, void* out_dev, cudaStream_t st, float* ms) {
-  hp_status s = ensure_device(tmp);
+  hp_status s = ensure_device(tmp, &st);
   if (s != HP_OK) return s;
   if ((s = run_rect(tmp, in_dev, out_dev, st)) != HP_OK) return s;  // warm-up (and launch configuration)
   float est = 0.0f;
@@ -196,7 +196,7 @@ hp_status time_plan(hp_nest* tmp, const void* const* in_dev, void* out_dev, cuda
 // outputs), so that a small nest is timed at the throughput it gets there
 hp_status time_plan_batched(hp_nest* tmp, const void* const* in_dev, void* out_dev, cudaStream_t st, int copies,
                             float* ms) {
-  hp_status s = ensure_device(tmp);
+  hp_status s = ensure_device(tmp, &st);
   if (s != HP_OK) return s;
   std::vector<hp_nest*> ns(copies, tmp);
   std::vector<const void* const*> ins(copies, in_dev);
@@ -268,9 +268,9 @@ hp_status tune_impl(hp_nest* n, const hp_level_req* req, const void* const* in_d
     }
     if (!any) return fail(HP_EINVAL, "no candidate map meets the level requirements (" + why + ")");
   }
-  hp_status s = ensure_device(n);
-  if (s != HP_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  hp_status s = ensure_device(n, &st);
+  if (s != HP_OK) return s;
   TuneKey key = tune_key(p);
   if (req) key.req = req_hash(p.depth, req);
   TuneChoice best;
@@ -368,7 +368,7 @@ hp_status tune_impl(hp_nest* n, const hp_level_req* req, const void* const* in_d
   if (s != HP_OK) return s;
   n->plan = np;
   n->plan_id = next_plan_id();   // cached batches built with the old plan no longer match
-  s = ensure_device(n);
+  s = ensure_device(n, &st);
   if (s != HP_OK) return s;
   return run_rect(n, in_dev, out_dev, st);  // the outputs hold the installed plan's result
 }
