@@ -642,8 +642,10 @@ struct CsrRun {
   hp_status bin() {
     const CsrPlan& p = n->csr;
     const CsrState& cs = *n->cs;
-    const int grid = static_cast<int>(
-        std::max<int64_t>(1, std::min<int64_t>((p.n_rows + kCsrThreads - 1) / kCsrThreads, 8 * n->sms)));
+    // enough CTAs for the rows and for the histogram's bins, which it clears (100 rows, 2^24
+    // bins: 2057 us with the rows' one CTA)
+    const int64_t most = std::max<int64_t>(p.n_rows, a.hist ? p.n_bins : 0);
+    const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((most + kCsrThreads - 1) / kCsrThreads, 8 * n->sms)));
     csr_bin_kernel<<<grid, kCsrThreads, 0, st>>>(a.off, p.n_rows, p.fixed_class, cs.counters, cs.rows01, cs.rows23,
                                                  cs.chunk_row, cs.chunk_idx, cs.chunk_cnt, cs.max_chunks, n->err, a.hist,
                                                  p.n_bins);
