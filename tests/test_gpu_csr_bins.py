@@ -1,5 +1,10 @@
 """GPU test of the fused histogram with many more bins than rows (its clear has to
-reach every bin, by more CTAs than the rows take): exact counts, run after run."""
+reach every bin, by more CTAs than the rows take): exact counts, run after run;
+and with as many as one CTA counts in shared memory, in a process's first nest."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -33,3 +38,35 @@ def test_more_bins_than_rows(rows, bins):
     # 2^24 bins are 134 MB: 20 us at HBM's rate, 2000 us by one CTA
     assert t0.elapsed_time(t1) < 0.5
     n.close()
+
+
+FIRST_NEST = """
+import torch
+from paper_2309_01906_gb300 import binding as hb
+s = torch.cuda.current_stream().cuda_stream
+g = torch.Generator("cuda").manual_seed(1)
+rows, ms = 400000, []
+off = torch.arange(rows + 1, device="cuda") * 40
+for bins in (12288, 12000):
+    col = torch.randint(0, bins, (rows * 40,), dtype=torch.int32, device="cuda", generator=g)
+    ins = [off, col, torch.ones(rows * 40, device="cuda"), torch.ones(bins, device="cuda"),
+           torch.empty(bins, dtype=torch.int64, device="cuda")]
+    y = torch.empty(rows, device="cuda")
+    n = hb.Nest(csr_rows=rows, red_level=1, op="sum", prec="f32_comp", body="csr_gather",
+                params=hb.hp_csr_params(rows * 40, bins, 0, 1, bins))
+    t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    for _ in range(20):
+        t0.record(); n.run([t.data_ptr() for t in ins], y.data_ptr(), s); t1.record(); t1.synchronize()
+        ms.append(t0.elapsed_time(t1))
+print(min(ms[:20]), min(ms[20:]))
+"""
+
+
+def test_the_first_nest_of_a_process_gets_its_ctas():
+    """The launch is sized after the kernel's shared memory is raised: 12288 bins take
+    a twentieth longer than 12000, with one CTA per SM 2.7 times as long."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_NEST], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    most, fewer = (float(v) for v in r.stdout.split())
+    assert most < 1.6 * fewer
