@@ -55,9 +55,13 @@ constexpr int64_t kCsrLimit0 = 4, kCsrLimit1 = HP_CSR_LIMIT1, kCsrLimit2 = HP_CS
 constexpr int64_t kCsrChunk = HP_CSR_CHUNK;
 static_assert(kCsrLimit3 >= kCsrChunk, "split rows must be longer than one chunk (bounds the chunk slots)");
 constexpr int kCsrThreads = 256;                          // every kernel's CTA
-// rows of one unit of work, by class: a chunk, a row, 4 rows per warp, 8 rows
-// per 8-lane team, 8 rows per thread
-constexpr int kCsrUnit0 = 8 * kCsrThreads, kCsrUnit1 = kCsrThreads, kCsrUnit2 = 4 * kCsrThreads / 32;
+// rows of one unit of work, by class: a chunk, a row, up to kCsrWarpRows rows per
+// warp, 8 rows per 8-lane team, 8 rows per thread
+constexpr int kCsrUnit0 = 8 * kCsrThreads, kCsrUnit1 = kCsrThreads, kCsrWarps = kCsrThreads / 32;
+// fewer where a CTA would not get 8 units (rows of 2000, 4 rows per warp and now: 5000
+// rows, 157 units for 760 CTAs, 119 and 56 us; 50,000, whose 1562 units leave a last
+// wave nearly empty, 446 and 379)
+constexpr int kCsrWarpRows = 4;
 // up to this many chunk slots the last CTA of the work kernel folds the long
 // rows' partials; beyond, a kernel of its own does (25,000 rows would take one
 // CTA about 200 us)
@@ -464,7 +468,7 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
   using Acc = typename Op::Acc;
   extern __shared__ int sh_hist[];
   __shared__ Acc wsh[2][kCsrThreads / 32];
-  __shared__ uint32_t s_unit, s_first[kCsrClasses], s_rows[3], s_end;
+  __shared__ uint32_t s_unit, s_first[kCsrClasses], s_rows[3], s_per, s_end;   // s_per: class 2's rows per warp
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned long long* const claim = reinterpret_cast<unsigned long long*>(&l.counters[kCntUnit]);
@@ -481,7 +485,10 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
     s_first[4] = 0;
     s_first[3] = static_cast<uint32_t>(slots);
     s_first[2] = s_first[3] + static_cast<uint32_t>(min(l.counters[3], l.n_rows));
-    s_first[1] = s_first[2] + (s_rows[2] + kCsrUnit2 - 1) / kCsrUnit2;
+    uint32_t per = kCsrWarpRows;
+    while (per > 1 && s_rows[2] < 8 * gridDim.x * (kCsrWarps * per)) per /= 2;
+    s_per = per;
+    s_first[1] = s_first[2] + (s_rows[2] + kCsrWarps * per - 1) / (kCsrWarps * per);
     s_first[0] = s_first[1] + (s_rows[1] + kCsrUnit1 - 1) / kCsrUnit1;
     s_end = s_first[0] + (s_rows[0] + kCsrUnit0 - 1) / kCsrUnit0;
   }
@@ -513,10 +520,9 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
         if (chunk) part[u] = r;
         else a.y[row] = Op::finish(r);
       }
-    } else if (u < s_first[1]) {   // 4 rows per warp; lane i reads the i-th one's place
-      constexpr int kRows = kCsrUnit2 / (kCsrThreads / 32);
-      const uint32_t k0 = (u - s_first[2]) * kCsrUnit2 + warp * kRows;
-      const int n = k0 >= s_rows[2] ? 0 : static_cast<int>(min(s_rows[2] - k0, static_cast<uint32_t>(kRows)));
+    } else if (u < s_first[1]) {   // s_per rows per warp; lane i reads the i-th one's place
+      const uint32_t per = s_per, k0 = ((u - s_first[2]) * kCsrWarps + warp) * per;
+      const int n = k0 >= s_rows[2] ? 0 : static_cast<int>(min(s_rows[2] - k0, per));
       int32_t id = 0;
       int64_t s = 0, e = 0;
       if (lane < n) {
