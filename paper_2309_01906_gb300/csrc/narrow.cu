@@ -315,11 +315,18 @@ __device__ __forceinline__ int32_t fold_range(const E* __restrict__ a, const E* 
 #pragma unroll
       for (int u = 0; u < 4; ++u) fold(q[u], r[u]);
     }
-    for (; n > 0; --n, ap += T, wq += T) {
-      const uint4 q = __ldcs(ap);
-      uint4 r = make_uint4(0u, 0u, 0u, 0u);
-      if constexpr (DOT) r = __ldg(wq);
-      fold(q, r);
+    if (n > 0) {   // the last one to three, in flight together
+      uint4 q[3], r[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const int64_t at = u < n ? u * T : 0;
+        q[u] = __ldcs(ap + at);
+        if constexpr (DOT) r[u] = __ldg(wq + at);
+        else r[u] = make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (u < n) fold(q[u], r[u]);
     }
   }
   return RAGGED ? Op::combine(acc, Op::value(run)) : Op::value(run);
@@ -334,6 +341,26 @@ __global__ void __launch_bounds__(kNarThreads, RAGGED ? (DOT ? 5 : 6) : kNarMinB
     const E* a = static_cast<const E*>(g.a) + o * g.R;
     const E* w = static_cast<const E*>(g.w);
     int32_t v = fold_range<E, OP, DOT, RAGGED>(a, w, 0, g.R, g.R, lane, 32);
+    v = Op::warp_reduce(v);
+    if (lane == 0) g.out[o] = v;
+  }
+}
+
+// a warp per row, one element per lane and load: ragged rows of a few hundred
+// elements, too few for the shared-warp kernel's start to pay (row_kernel)
+template <class E, int OP, bool DOT>
+__global__ void __launch_bounds__(kNarThreads, kNarMinBlocks) narrow_elements_kernel(NarArgs g) {
+  using Op = NarrowOp<E, OP>;
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = static_cast<int64_t>(gridDim.x) * (kNarThreads / 32);
+  const E* w = static_cast<const E*>(g.w);
+  for (int64_t o = static_cast<int64_t>(blockIdx.x) * (kNarThreads / 32) + (threadIdx.x >> 5); o < g.O; o += warps) {
+    const E* a = static_cast<const E*>(g.a) + o * g.R;
+    int32_t v = Op::ident();
+    for (int64_t x = lane; x < g.R; x += 32) {
+      const int32_t e = static_cast<int32_t>(a[x]);
+      v = Op::combine(v, DOT ? e * static_cast<int32_t>(w[x]) : e);
+    }
     v = Op::warp_reduce(v);
     if (lane == 0) g.out[o] = v;
   }
@@ -526,9 +553,33 @@ int short_lanes(int granules) {
   return best;
 }
 
+// Which kernel takes the rows of a warp team?  The shared-warp kernel
+// (narrow_rows_kernel) folds the most rows per second, but its start (tables in
+// shared memory, several rounds of granules per lane) costs about a microsecond,
+// two and a half with the tables of a ragged dot product, which only many rows
+// earn back.  Device times of 1000 and 30,000 rows, the shared-warp kernel / a warp
+// per row: 64 bytes 2.7 / 1.4 and 2.7 / 4.4 us, 16 bytes 1.6 / 1.4 and 1.6 / 4.3; ragged
+// 1000 bytes 3.9 / 1.8 and 6.8 / 9.8; ragged 100 bytes, with a warp per row by elements,
+// 3.6 / 1.4 and 3.6 / 4.5, dot product 5.8 / 1.5 and 5.8 / 5.3.
+enum RowKernel { ROW_WARP, ROW_SHARED, ROW_ELEMENTS };
+RowKernel row_kernel(const NarrowPlan& p, bool ragged, int sms) {
+  const int64_t bytes = p.R * p.esize;
+  if (p.R < 1 || bytes > (ragged ? kShortBytes : kShortAligned)) return ROW_WARP;
+  if (!ragged) return p.O > (bytes <= 32 ? 20 : bytes <= 256 ? 80 : 100) * static_cast<int64_t>(sms) ? ROW_SHARED : ROW_WARP;
+  // beyond about 12 elements per lane whole pieces beat single elements; a warp per row fills
+  // the SMs once with 48 to 64 rows each
+  if (p.R > 384) return p.O > 80 * static_cast<int64_t>(sms) ? ROW_SHARED : ROW_WARP;
+  // the start against what a thousand rows take longer by elements (measured lines, us)
+  const bool dot = p.body == HP_BODY_DOT_BCAST;
+  const double start = dot ? 3.4 : bytes <= 16 ? 0.95 : 1.8;
+  const double elements = 0.09 + (dot ? 0.0003 : 0.00015) * p.R, shared = (dot ? 0.00029 : 0.00017) * bytes;
+  return p.O / 1000.0 * (elements - shared) * (152.0 / sms) > start ? ROW_SHARED : ROW_ELEMENTS;
+}
+
 template <class E, int OP, bool DOT, bool RAGGED>
 cudaError_t launch_narrow(const NarrowPlan& p, const NarArgs& g, int sms, cudaStream_t st) {
-  if (p.team == 0 && p.R > 0 && p.R * p.esize <= (RAGGED ? kShortBytes : kShortAligned)) {
+  const RowKernel rows = p.team == 0 ? row_kernel(p, RAGGED, sms) : ROW_WARP;
+  if (rows == ROW_SHARED) {
     const int bytes = static_cast<int>(p.R) * p.esize;
     const int L = short_lanes(RAGGED ? (bytes + 30) / 16 : bytes / 16);
     auto k = narrow_rows_kernel<E, OP, DOT, RAGGED>;
@@ -537,6 +588,9 @@ cudaError_t launch_narrow(const NarrowPlan& p, const NarArgs& g, int sms, cudaSt
   } else if (p.team == 0) {
     const int64_t need = ceil_div64(p.O, kNarThreads / 32);
     auto k = narrow_warp_kernel<E, OP, DOT, RAGGED>;
+    if constexpr (RAGGED) {
+      if (rows == ROW_ELEMENTS) k = narrow_elements_kernel<E, OP, DOT>;
+    }
     k<<<static_cast<int>(balanced_grid(need, nar_blocks(k, kNarThreads, sms))), kNarThreads, 0, st>>>(g);
   } else {
     const int threads = 32 * p.W;
