@@ -27,6 +27,7 @@
 #include <cmath>
 #include <sstream>
 #include <string>
+#include <type_traits>
 
 #include "api_internal.h"
 
@@ -177,7 +178,7 @@ struct OrdArgs {
   float* part;        // the state of every (output, part) when G > 1
   int32_t* tickets;   // per output, G > 1
   int64_t O, R, G, part_len, chunk;
-  int64_t total;      // iterations of the whole nest, O * R
+  int64_t total;      // iterations of the whole nest, O * R; 0: no shifted granules
   int32_t W;
 };
 
@@ -185,8 +186,11 @@ struct OrdArgs {
 // that hold them, and a shift by the start's place in the first (the same in
 // every lane of a warp, whose pieces are 32 bytes apart).  Scalar loads of a
 // lane's own piece take eight requests for what one 256-bit load brings (33520
-// rows of 1001 maps: 71 us, 50 so).  granules() only loads, so that two arrays'
-// loads overlap; shift() selects.
+// rows of 1001 maps: 71 us, 50 so).  load() only loads, so that two arrays'
+// loads overlap; shift() selects, which takes a lone warp longer than the requests:
+// few rows that are short, up to 3 rows, and rows of fewer than 8 iterations keep the
+// scalar loads (one row of 1001 maps: 3.3 us so, 4.1 with granules; 10 rows 4.4 and 4.1;
+// 10 rows of 50: 1.7 and 1.9).
 struct Granules {
   float4 a, b, c;
   uint32_t m;
@@ -205,6 +209,11 @@ struct Granules {
     for (int k = 0; k < 8; ++k) r[k] = (m & 1u) ? v[k + 1] : v[k];
   }
 };
+// Ragged rows of one round of a warp read a last, shorter piece like the others, so
+// that its lane does not keep the rest waiting (1000 rows of 31 maps: 2.3 us with a loop of
+// its own, 2.0 so); a form of its own, since in longer rows it costs every round and more
+// registers (5000 rows of 3001: 30.9 us and 33.4).
+constexpr int64_t kOneRound = 32 * 8;
 // Is every granule of the piece at index i inside an array of n?
 __device__ __forceinline__ bool granules_inside(int64_t i, int64_t n) { return i >= 4 && i + 12 <= n; }
 
@@ -217,8 +226,9 @@ __device__ __forceinline__ void ld8(const float* p, float* r) {
 
 // A lane walks its own block, so its loads do not coalesce across the warp:
 // V = 8 takes whole 32-byte sectors with 256-bit loads (each in one request),
-// V = 4 128-bit loads, V = 1 shifted granules (whole pieces) and scalar loads.  Every fold runs over [s, e) of the
-// output whose first iteration is `base`, in order.
+// V = 4 128-bit loads, V = 1 shifted granules or scalar loads, and V = 2 those in
+// rows of one round (kOneRound).  Every fold runs over [s, e) of the output whose
+// first iteration is `base`, in order.
 
 struct AffineOp {
   using S = float2;   // (A, B)
@@ -241,7 +251,8 @@ struct AffineOp {
 
 template <int V>
 __device__ __forceinline__ float2 fold_affine(const float* __restrict__ a, const float* __restrict__ b, int64_t s,
-                                            int64_t e, int64_t total, float2 v) {
+                                            int64_t e, float2 v) {
+  static_assert(V == 8 || V == 4, "whole vectors");
   if constexpr (V == 8) {
     for (; s + 16 <= e; s += 16) {
       float av[16], bv[16];
@@ -259,7 +270,7 @@ __device__ __forceinline__ float2 fold_affine(const float* __restrict__ a, const
 #pragma unroll
       for (int q = 0; q < 8; ++q) v = AffineOp::combine(v, make_float2(av[q], bv[q]));
     }
-  } else if constexpr (V == 4) {
+  } else {
     for (; s + 16 <= e; s += 16) {   // four 128-bit loads of each input in flight
       float4 av[4], bv[4];
 #pragma unroll
@@ -283,10 +294,47 @@ __device__ __forceinline__ float2 fold_affine(const float* __restrict__ a, const
       v = AffineOp::combine(v, make_float2(a0.z, b0.z));
       v = AffineOp::combine(v, make_float2(a0.w, b0.w));
     }
+  }
+  return v;
+}
+
+// at any alignment; s and e count from the arrays' start
+__device__ __forceinline__ float2 fold_affine_any(const float* __restrict__ a, const float* __restrict__ b, int64_t s,
+                                                int64_t e, int64_t total, float2 v) {
+  for (; s + 8 <= e; s += 8) {
+    float av[8], bv[8];
+    if (granules_inside(s, total)) {
+      Granules ga, gb;
+      ga.load(a + s);
+      gb.load(b + s);
+      ga.shift(av);
+      gb.shift(bv);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        av[q] = __ldg(a + s + q);
+        bv[q] = __ldg(b + s + q);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v = AffineOp::combine(v, make_float2(av[q], bv[q]));
+  }
+  for (; s < e; ++s) v = AffineOp::combine(v, make_float2(__ldg(a + s), __ldg(b + s)));
+  return v;
+}
+
+template <int V>
+__device__ __forceinline__ AffineOp::S AffineOp::fold(const OrdArgs& g, int64_t base, int64_t s, int64_t e, S v) {
+  if constexpr (V >= 4) {
+    return fold_affine<V>(g.a + base, g.b + base, s, e, v);
+  } else if constexpr (V == 1) {
+    return fold_affine_any(g.a, g.b, base + s, base + e, g.total, v);
   } else {
-    for (; s + 8 <= e; s += 8) {
-      float av[8], bv[8];
-      if (granules_inside(s, total)) {
+    const float *__restrict__ a = g.a + base, *__restrict__ b = g.b + base;
+    float av[8], bv[8];
+    for (; s < e; s += 8) {
+      const int n = e - s < 8 ? static_cast<int>(e - s) : 8;
+      if (granules_inside(base + s, g.total)) {
         Granules ga, gb;
         ga.load(a + s);
         gb.load(b + s);
@@ -295,22 +343,16 @@ __device__ __forceinline__ float2 fold_affine(const float* __restrict__ a, const
       } else {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          av[q] = __ldg(a + s + q);
-          bv[q] = __ldg(b + s + q);
+          av[q] = q < n ? __ldg(a + s + q) : 0.0f;
+          bv[q] = q < n ? __ldg(b + s + q) : 0.0f;
         }
       }
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v = AffineOp::combine(v, make_float2(av[q], bv[q]));
+      for (int q = 0; q < 8; ++q)
+        if (q < n) v = combine(v, make_float2(av[q], bv[q]));
     }
-    for (; s < e; ++s) v = AffineOp::combine(v, make_float2(__ldg(a + s), __ldg(b + s)));
+    return v;
   }
-  return v;
-}
-
-template <int V>
-__device__ __forceinline__ AffineOp::S AffineOp::fold(const OrdArgs& g, int64_t base, int64_t s, int64_t e, S v) {
-  if constexpr (V == 1) return fold_affine<V>(g.a, g.b, base + s, base + e, g.total, v);
-  else return fold_affine<V>(g.a + base, g.b + base, s, e, g.total, v);
 }
 
 struct Mat2Op {
@@ -378,7 +420,7 @@ struct LastOp {
   // shifted granules: the smaller piece keeps a warp's requests to a few lines
   // each (the result is exact whatever the pieces)
   template <int V>
-  __host__ __device__ static constexpr int64_t piece() { return V == 1 ? 8 : 32; }
+  __host__ __device__ static constexpr int64_t piece() { return V < 4 ? 8 : 32; }
   __device__ static S ident() { return __int_as_float(0x7fc00000); }
   __device__ static S combine(S e, S l) { return l != l ? e : l; }
   __device__ static S shfl(S v, int m) { return __shfl_down_sync(0xffffffffu, v, m); }
@@ -418,7 +460,7 @@ struct LastOp {
         const float4 q = __ldg(reinterpret_cast<const float4*>(a + s));
         v = combine(combine(combine(combine(v, q.x), q.y), q.z), q.w);
       }
-    } else {
+    } else if constexpr (V == 1) {
       for (; s + 8 <= e; s += 8) {
         float r[8];
         if (granules_inside(base + s, g.total)) {
@@ -433,6 +475,22 @@ struct LastOp {
         for (int q = 0; q < 8; ++q) v = combine(v, r[q]);
       }
       for (; s < e; ++s) v = combine(v, __ldg(a + s));
+    } else {
+      float r[8];
+      for (; s < e; s += 8) {
+        const int n = e - s < 8 ? static_cast<int>(e - s) : 8;
+        if (granules_inside(base + s, g.total)) {
+          Granules gr;
+          gr.load(a + s);
+          gr.shift(r);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) r[q] = q < n ? __ldg(a + s + q) : 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (q < n) v = combine(v, r[q]);
+      }
     }
     return v;
   }
@@ -553,11 +611,24 @@ int out_floats(const OrderedPlan& p) {
   return p.op == HP_RED_MAT2_PRODUCT ? Mat2Op::kOut : (p.op == HP_RED_LAST_VALID ? LastOp::kOut : AffineOp::kOut);
 }
 
+// Lanes per row of a warp team whose lanes take pieces of `piece` iterations (32: a
+// warp each).  Rows of more than one piece or 16 iterations share a warp once there
+// are more of them than the SMs take warps at once: below, fewer warps only make
+// each one's loads more (100 values, 1000 rows: 1.9 us with a warp each, 2.4 shared;
+// 10,000 rows 4.9 and 3.0).  16 lanes of 32 values share nothing worth it (30,000
+// rows of 500: 15.3 with a warp each, 17.0 shared).
+constexpr int64_t kOrdSharedRows = 18;   // rows per SM
+int row_lanes(const OrderedPlan& p, int64_t piece, int sms) {
+  int L = 32;
+  while (L > 1 && L / 2 * piece >= p.R) L /= 2;
+  const int64_t few = L <= 2 ? 12 : L <= 8 ? kOrdSharedRows : 24;
+  return (L > 1 || p.R > 16) && (p.O <= few * sms || L * piece > 256) ? 32 : L;
+}
+
 template <class Op, int V>
 void launch_ordered(const OrderedPlan& p, const OrdArgs& g, int sms, cudaStream_t st) {
-  if (p.team == 0) {
-    int L = 32;
-    while (L > 1 && L / 2 * Op::template piece<V>() >= p.R) L /= 2;
+  if (V == 2 || p.team == 0) {
+    const int L = row_lanes(p, Op::template piece<V>(), sms);
     const int64_t need = ceil_div(p.O, static_cast<int64_t>(kOrdThreads) / L);
     if (L < 32) {
       auto k = ordered_short_kernel<Op, V>;
@@ -566,21 +637,21 @@ void launch_ordered(const OrderedPlan& p, const OrdArgs& g, int sms, cudaStream_
       auto k = ordered_warp_kernel<Op, V>;
       k<<<static_cast<int>(balanced_grid(need, blocks_for(k, kOrdThreads, sms))), kOrdThreads, 0, st>>>(g);
     }
-  } else {
+  } else if constexpr (V != 2) {
     const int threads = 32 * p.W;
-    auto go = [&](auto k) {
-      const int grid = static_cast<int>(balanced_grid(p.O * p.G, blocks_for(k, threads, sms)));
-      k<<<grid, threads, 0, st>>>(g);
-    };
-    go(ordered_block_kernel<Op, V>);
+    auto k = ordered_block_kernel<Op, V>;
+    k<<<static_cast<int>(balanced_grid(p.O * p.G, blocks_for(k, threads, sms))), threads, 0, st>>>(g);
   }
 }
 
 template <class Op>
 void launch_ordered_v(const OrderedPlan& p, const OrdArgs& g, int v, int sms, cudaStream_t st) {
-  if (v == 8) launch_ordered<Op, 8>(p, g, sms, st);
-  else if (v == 4) launch_ordered<Op, 4>(p, g, sms, st);
-  else launch_ordered<Op, 1>(p, g, sms, st);
+  if (v == 8) return launch_ordered<Op, 8>(p, g, sms, st);
+  if (v == 4) return launch_ordered<Op, 4>(p, g, sms, st);
+  if constexpr (!std::is_same_v<Op, Mat2Op>) {
+    if (p.team == 0 && p.R >= 8 && p.R <= kOneRound) return launch_ordered<Op, 2>(p, g, sms, st);
+  }
+  launch_ordered<Op, 1>(p, g, sms, st);
 }
 
 }  // namespace
@@ -619,7 +690,8 @@ hp_status run_ordered(hp_nest* n, const void* const* in_dev, void* out_dev, cuda
   g.G = p.G;
   g.part_len = std::max<int64_t>(p.part, 1);
   g.chunk = p.chunk;
-  g.total = p.O * p.R;
+  const bool granules = p.R >= 64 ? p.O >= 4 || p.R > 2048 : p.R >= 8 && p.O > kOrdSharedRows * n->sms;
+  g.total = granules ? p.O * p.R : 0;
   g.W = p.W;
   if (reinterpret_cast<uintptr_t>(out_dev) % 4 != 0) return fail(HP_EINVAL, "out must be 4-byte aligned");
   // the widest loads the plan and the input alignment allow (blocks start at whole loads)
