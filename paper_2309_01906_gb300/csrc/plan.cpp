@@ -189,7 +189,11 @@ static void auto_map(const NestPlan& p, hp_level_map* m) {
   int red_hw;
   int sub = 0;
   if (R >= 4096) {
-    red_hw = (O < 12 * kAssumedSMs && R >= 65536 && grid_parts(O, R) > 1) ? HP_HW_GRID : HP_HW_CTA;
+    // From two outputs per SM on a CTA each: splitting them too gains single runs of up to
+    // three per SM some (304 x 65536 FP32 9.0 us split, 11.2 not; 500 x 65536 18.4 and 17.3), but
+    // costs the batched executor a ticket per part (27 us split, 21 not; 80 and 69 for
+    // three of 500 x 65536) and needs scratch.
+    red_hw = (O < 2 * kAssumedSMs && R >= 65536) ? HP_HW_GRID : HP_HW_CTA;
   } else if (R >= 512) {
     red_hw = HP_HW_WARP;
   } else if (R >= 32) {

@@ -41,7 +41,7 @@ def test_one_nest_listed_many_times():
     import torch
     s = torch.cuda.current_stream().cuda_stream
     g = torch.Generator("cuda").manual_seed(4)
-    for O, R, level_map in [(400, 65536, None), (1, 1 << 20, None), (7, 5000, ["grid", ("grid", 0, 625)])]:
+    for O, R, level_map in [(300, 65536, None), (1, 1 << 20, None), (7, 5000, ["grid", ("grid", 0, 625)])]:
         n = hb.Nest([O, R], 1, "sum", "i64", "load", level_map=level_map)
         assert n.describe()["grid_parts"] > 1
         ins = [torch.randint(-(1 << 30), 1 << 30, (O, R), dtype=torch.int32, device="cuda", generator=g) for _ in range(8)]
