@@ -170,6 +170,7 @@ hp_status plan_rect(int depth, const int64_t* extents, const hp_level_map* map, 
                     hp_prec prec, hp_body body, const void* body_params, NestPlan* out, std::string* why);
 
 std::string describe_plan(const NestPlan& p);
+int64_t counted_items(const NestPlan& p);   // items whose partials a memory budget counts
 
 // A-priori bound on |got - exact| / sum|t| for one FP result of the plan.
 double error_bound_rect(const NestPlan& p);

@@ -136,6 +136,15 @@ static int64_t grid_parts(int64_t O, int64_t n) {
   return best;
 }
 
+// An automatic map may cut more parts than give every SM its teams, to spread them
+// evenly.  A server's budget does not count those (their scratch is its pool's), so
+// that the spreading refuses no request.
+int64_t counted_items(const NestPlan& p) {
+  const int64_t O = p.rp.O;
+  if (!p.auto_map || p.tuned || O < 1) return p.rp.items;
+  return std::min(p.rp.items, O * ((HP_PLAN_TEAMS_PER_SM * kAssumedSMs + O - 1) / O));
+}
+
 static void auto_map(const NestPlan& p, hp_level_map* m);
 
 // outputs over the grid; every reduced level on the chosen hardware level

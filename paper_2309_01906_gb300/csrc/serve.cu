@@ -215,6 +215,7 @@ struct hp_server {
 namespace hp {
 namespace {
 
+// a request's bytes against the budget: inputs, outputs and scratch
 size_t request_bytes(const hp_nest* n, size_t* part_bytes, size_t* ticket_bytes) {
   const NestPlan& p = n->plan;
   const RectPlan& rp = p.rp;
@@ -223,7 +224,8 @@ size_t request_bytes(const hp_nest* n, size_t* part_bytes, size_t* ticket_bytes)
   b += static_cast<size_t>(rp.O) * p.out_elem_bytes;
   *part_bytes = rp.G > 1 ? static_cast<size_t>(rp.items) * partial_bytes(p.prec, p.op) : 0;
   *ticket_bytes = rp.G > 1 ? static_cast<size_t>(rp.O) * sizeof(int32_t) : 0;
-  return b + *part_bytes + *ticket_bytes;
+  const size_t scratch = rp.G > 1 ? static_cast<size_t>(counted_items(p)) * partial_bytes(p.prec, p.op) : 0;
+  return b + scratch + *ticket_bytes;
 }
 
 // tiles of one request's nest (work items cut into ranges of about `target` elements)
