@@ -97,7 +97,7 @@ struct LaunchCfg {
   int threads = 0;     // per CTA
   int cluster = 1;     // CTAs per cluster
   int M = 1;           // items per round of a block team
-  int rows = 0;        // the rows kernel this geometry is for (RowsKind; 0: none)
+  int rows_grid[2] = {0, 0};   // CTAs of the rows kernels (RowsKind - 1): an input's alignment picks the kernel
 };
 
 // Plan of a nest with an ordered (non-commutative) reduction: outputs over the

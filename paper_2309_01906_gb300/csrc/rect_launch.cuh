@@ -45,7 +45,7 @@ RowsKind rows_kind(const RectPlan& rp, const void* A) {
   return rp.L > 1 || rp.R < 5 ? ROWS_TEAM : ROWS_NONE;
 }
 
-// launch of a rows kernel; cfg is filled on the nest's first run of that kind
+// launch of a rows kernel; its grid is sized on the nest's first run of that kind
 template <class Op, int V, bool DOT>
 hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const typename Op::In* A,
                       const typename Op::In* w, const RectArgs& a) {
@@ -56,7 +56,8 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
   auto kt = K > 1 ? rect_thread_rows_kernel<Op, V, DOT, true> : rect_thread_rows_kernel<Op, V, DOT, false>;
   const size_t dyn = kind == ROWS_THREAD ? sizeof(int32_t) * (kRowsThreads / 32) * kThreadRowsStages * set * K * rp.R : 0;
   const int U = rp.L == 1 ? kRowsU : 1;
-  if (!cfg.ready || cfg.rows != kind) {
+  int& grid = cfg.rows_grid[kind - 1];
+  if (grid == 0) {
     const void* f = kind == ROWS_THREAD ? reinterpret_cast<const void*>(kt)
                     : U == 1            ? reinterpret_cast<const void*>(k1)
                                         : reinterpret_cast<const void*>(k4);
@@ -71,19 +72,17 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
     if (per_sm < 1) return fail(HP_EUNSUPPORTED, "kernel does not fit on an SM with this CTA size");
     const int64_t cta_rows = static_cast<int64_t>(kRowsThreads / 32) * set * (kind == ROWS_THREAD ? K : U);
     const int64_t blocks = std::min<int64_t>((rp.O + cta_rows - 1) / cta_rows, static_cast<int64_t>(per_sm) * cfg.sms);
-    cfg.threads = kRowsThreads;
-    cfg.grid = static_cast<int>(std::max<int64_t>(blocks, 1));
-    cfg.rows = kind;
+    grid = static_cast<int>(std::max<int64_t>(blocks, 1));
     cfg.ready = true;
   }
   if (rp.O == 0) return HP_OK;
   Out* out = static_cast<Out*>(a.out);
   if (kind == ROWS_THREAD) {
-    kt<<<cfg.grid, kRowsThreads, dyn, a.stream>>>(rp.O, static_cast<int>(rp.R), rp.L, K, A, w, out, a.comp);
+    kt<<<grid, kRowsThreads, dyn, a.stream>>>(rp.O, static_cast<int>(rp.R), rp.L, K, A, w, out, a.comp);
   } else {
     const RowsArgs g{rp.O, static_cast<int32_t>(rp.R), rp.vP[0], rp.L, rp.grp_lanes, rp.cg[0], rp.cl[0]};
-    if (U == 1) k1<<<cfg.grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
-    else k4<<<cfg.grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
+    if (U == 1) k1<<<grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
+    else k4<<<grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
   }
   const cudaError_t e = cudaPeekAtLastError();
   return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_rows_kernel launch");
@@ -117,7 +116,7 @@ template <class Op, int V, bool DOT>
 hp_status launch_flat(const RectPlan& rp, LaunchCfg& cfg, const typename Op::In* A, const typename Op::In* w,
                       const RectArgs& a) {
   auto k = rect_flat_kernel<Op, V, DOT>;
-  if (!cfg.ready) {
+  if (cfg.grid == 0) {
     cfg.threads = 32 * rp.W;
     int per_sm = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, cfg.threads, 0);
@@ -146,7 +145,7 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
   rp.comp = a.comp;
   if (rp.team == TEAM_MAP) {
     auto k = rect_map_kernel<Op, Body>;
-    if (!cfg.ready) {
+    if (cfg.grid == 0) {
       cfg.threads = 256;
       const int64_t blocks = (rp.O + 255) / 256;
       cfg.grid = static_cast<int>(blocks < 8LL * cfg.sms ? (blocks > 0 ? blocks : 1) : 8LL * cfg.sms);
@@ -176,8 +175,7 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
       pipe ? static_cast<size_t>(32 * rp.W) *
                  std::max<size_t>(pipe_depth(rp.groups) * rp.groups * 16, kPatMax * sizeof(int32_t))
            : 0;
-  if (!cfg.ready || cfg.rows != ROWS_NONE) {
-    cfg.rows = ROWS_NONE;
+  if (cfg.grid == 0) {
     cfg.threads = 32 * rp.W;
     cfg.cluster = block ? rp.C : 1;
     if (pipe) {
