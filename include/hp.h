@@ -362,7 +362,11 @@ hp_status hp_nest_tune(hp_nest *n, const void *const *in_dev, void *out_dev, voi
 hp_status hp_nest_error_bound(const hp_nest *n, double *rel_bound);
 
 /* Write the plan as one line of JSON (levels, hardware binding, team, grid,
- * vector width, kernels) into buf[len]; truncated if too small. */
+ * vector width) and the kernel that runs it into buf[len]; truncated if too
+ * small.  The kernel is the one for inputs that start on 16 bytes (plans of "vec" 1 take
+ * others too, which may go to another kernel) on a GPU of 152 SMs; "pipe" is
+ * the plan's: LOAD reductions of 4096 or more contiguous elements, 64-bit
+ * comparisons excepted, leave the pipeline for rect_flat. */
 hp_status hp_nest_describe(const hp_nest *n, char *buf, size_t len);
 
 /* Wait for the stream, then read the nest's device error word (0 = none;
@@ -627,7 +631,9 @@ void hp_stencil_destroy(hp_stencil *s);
  * Process-wide planner options, read when a nest is created (existing nests
  * keep their plan).  Names:
  *   "pipeline"  1 (default): block teams whose element groups allow it stream
- *               their inputs through per-thread cp.async rings; 0: plain loads.
+ *               their inputs through per-thread cp.async rings (single nests:
+ *               but for LOAD reductions of 4096 or more contiguous elements that
+ *               are not 64-bit comparisons); 0: plain loads.
  *               Both give bit-identical results (same reduction tree).
  *   "serve_batching"  1 (default): servers pack admitted requests into
  *               batched steps; 0: servers launch each request alone.

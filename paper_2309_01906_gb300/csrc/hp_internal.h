@@ -74,7 +74,7 @@ struct NestPlan {
   size_t in_elem_bytes = 4;
   size_t out_elem_bytes = 4;
   std::vector<float> geo_table;      // GEOMETRIC body values fl32(q^k), k < m
-  std::string kernel;                // name of the kernel family the plan runs
+  std::string kernel;                // the kernel that runs the plan (inputs on 16 bytes)
   bool tuned = false;                // map taken from the tuning cache
 };
 

@@ -131,9 +131,16 @@ hp_status plan_narrow(int depth, const int64_t* extents, const hp_level_map* map
   return HP_OK;
 }
 
+namespace {
+// which kernel takes the rows of a warp team (row_kernel)
+enum RowKernel { ROW_WARP, ROW_SHARED, ROW_ELEMENTS };
+RowKernel row_kernel(const NarrowPlan& p, bool ragged, int sms);
+}  // namespace
+
 std::string describe_narrow(const NarrowPlan& p) {
   static const char* hw[] = {"grid", "cluster", "cta", "warp", "subwarp", "lane", "seq", "auto"};
   static const char* ops[] = {"sum", "max", "min"};
+  static const char* kRowNames[] = {"warp", "rows", "elements"};
   std::ostringstream s;
   s << "{\"kind\":\"narrow\",\"prec\":\"" << (p.prec == HP_I8 ? "i8" : "i16") << "\",\"op\":\"" << ops[p.op]
     << "\",\"body\":\"" << (p.body == HP_BODY_LOAD ? "load" : "dot_bcast") << "\",\"depth\":" << p.depth
@@ -146,7 +153,7 @@ std::string describe_narrow(const NarrowPlan& p) {
   s << "],\"auto_map\":" << (p.auto_map ? "true" : "false") << ",\"team\":\"" << (p.team ? "block" : "warp")
     << "\",\"outputs\":" << p.O << ",\"reduced\":" << p.R << ",\"warps\":" << p.W << ",\"grid_parts\":" << p.G
     << ",\"part\":" << p.part << ",\"vec\":" << 16 / p.esize << ",\"simd\":" << 4 / p.esize << ",\"kernel\":\"narrow_"
-    << (p.team ? "block" : "warp") << "\"}";
+    << (p.team ? "block" : kRowNames[row_kernel(p, p.R % (16 / p.esize) != 0, 152)]) << "\"}";
   return s.str();
 }
 
@@ -561,7 +568,6 @@ int short_lanes(int granules) {
 // per row: 64 bytes 2.7 / 1.4 and 2.7 / 4.4 us, 16 bytes 1.6 / 1.4 and 1.6 / 4.3; ragged
 // 1000 bytes 3.9 / 1.8 and 6.8 / 9.8; ragged 100 bytes, with a warp per row by elements,
 // 3.6 / 1.4 and 3.6 / 4.5, dot product 5.8 / 1.5 and 5.8 / 5.3.
-enum RowKernel { ROW_WARP, ROW_SHARED, ROW_ELEMENTS };
 RowKernel row_kernel(const NarrowPlan& p, bool ragged, int sms) {
   const int64_t bytes = p.R * p.esize;
   if (p.R < 1 || bytes > (ragged ? kShortBytes : kShortAligned)) return ROW_WARP;

@@ -150,9 +150,14 @@ hp_status plan_ordered(int depth, const int64_t* extents, const hp_level_map* ma
   return HP_OK;
 }
 
+namespace {
+int row_lanes(const OrderedPlan& p, int64_t piece, int sms);
+}
+
 std::string describe_ordered(const OrderedPlan& p) {
   static const char* hw[] = {"grid", "cluster", "cta", "warp", "subwarp", "lane", "seq", "auto"};
   std::ostringstream s;
+  const int64_t piece = p.op == HP_RED_MAT2_PRODUCT ? 4 : p.op == HP_RED_LAST_VALID && p.V >= 4 ? 32 : 8;   // of aligned inputs
   const char* op = p.op == HP_RED_MAT2_PRODUCT ? "mat2_product" : (p.op == HP_RED_LAST_VALID ? "last_valid" : "affine_compose");
   s << "{\"kind\":\"ordered\",\"op\":\"" << op << "\",\"depth\":" << p.depth << ",\"red_level\":" << p.red_level
     << ",\"extents\":[";
@@ -165,7 +170,7 @@ std::string describe_ordered(const OrderedPlan& p) {
     << "\",\"outputs\":" << p.O << ",\"reduced\":" << p.R << ",\"warps\":" << p.W << ",\"grid_parts\":" << p.G
     << ",\"part\":" << p.part << ",\"chunk\":" << p.chunk << ",\"piece\":" << p.piece << ",\"vec\":" << p.V
     << ",\"chain\":" << p.k
-    << ",\"kernel\":\"ordered_" << (p.team ? "block" : "warp") << "\"}";
+    << ",\"kernel\":\"ordered_" << (p.team ? "block" : row_lanes(p, piece, 152) < 32 ? "short" : "warp") << "\"}";
   return s.str();
 }
 

@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include "hp_internal.h"
+#include "rect_route.h"
 
 namespace hp {
 
@@ -549,6 +550,8 @@ hp_status plan_rect(int depth, const int64_t* extents, const hp_level_map* map, 
   p.kernel = team_block ? (rp.pipe ? (rp.C > 1 ? "rect_block_pipe_cluster" : "rect_block_pipe")
                                    : (rp.C > 1 ? "rect_block_cluster" : "rect_block"))
                         : "rect_lanes";
+  if (rows_kind(p, true) != ROWS_NONE) p.kernel = rows_kind(p, true) == ROWS_THREAD ? "rect_thread_rows" : "rect_rows";
+  else if (flat_plan(p)) p.kernel = "rect_flat";
   *out = p;
   return HP_OK;
 }

@@ -21,6 +21,7 @@
 #include <cooperative_groups.h>
 #include <cstdint>
 
+#include "rect_route.h"
 #include "accum.cuh"
 #include "hp_internal.h"
 
@@ -589,7 +590,6 @@ struct RowsArgs {
   int32_t grp_lanes, cg, cl;   // slot of lane lt: (lt / grp_lanes) * cg + (lt % grp_lanes) * cl
 };
 constexpr int kRowsThreads = 256;
-constexpr int64_t kRowsMaxR = int64_t(1) << 22;   // 32-bit offsets within a warp's rows
 
 // the U rows' values at one position, folded into their accumulators
 template <class Op, int V, bool DOT, int U>
@@ -782,7 +782,6 @@ struct FlatArgs {
   int32_t G, P, W;
   int32_t grp_lanes, cw, cg, cl;
 };
-constexpr int kFlatThreads = 256;
 // CTAs per SM (swept): the dot product's second operand takes the registers of
 // one more load per position (600 x 2^18 compensated: 4 CTAs 101 us, 5 107, 6
 // 125); scalar loads need the most threads (20011 x 8195 int64: 8 CTAs 98 us, 6
@@ -874,7 +873,6 @@ __global__ void __launch_bounds__(kFlatThreads, (flat_blocks<Op, V, DOT>()))
 // here for dot products on two-word accumulators only, whose four rows a thread
 // take too many registers in rect_rows_kernel (compensated 64 us there, 48 here;
 // f32 29 and 33).
-constexpr int kThreadRowsMin = 5, kThreadRowsMax = 64;
 constexpr int kThreadRowsStages = 3;
 constexpr int kThreadRowsElems = 736;
 // sets of rows in a block: at least 16 warps' blocks for every SM

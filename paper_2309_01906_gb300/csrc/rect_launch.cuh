@@ -26,25 +26,6 @@ inline hp_status cuda_fail(cudaError_t e, const char* what) {
   return fail(HP_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// Which kernel folds whole rows (rect_rows_kernel, rect_thread_rows_kernel)?
-enum RowsKind { ROWS_NONE = 0, ROWS_TEAM = 1, ROWS_THREAD = 2 };
-template <class Op, bool DOT>
-RowsKind rows_kind(const RectPlan& rp, const void* A) {
-  if (rp.team != TEAM_LANES || rp.nv != 1 || rp.vstride[0] != 1 || rp.G != 1 || rp.split || rp.R < 1 || rp.R > kRowsMaxR)
-    return ROWS_NONE;
-  // one or two lanes a row: blocks of 32 rows are copied 16 bytes at a time
-  const bool aligned = (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
-  constexpr bool kWide = sizeof(typename Op::Acc) == 8, kComp = std::is_same_v<typename Op::Acc, f2>;
-  // vectors of plain rows from 16 elements on load whole sectors anyway (2^25
-  // elements in rows of 16, int64: 27 us in rect_lanes_kernel, 28 through shared memory)
-  const bool sectors = rp.V == 4 && rp.R >= 16 && !DOT && !kComp;
-  if (rp.R >= (kWide && DOT && rp.V == 4 ? 4 : kThreadRowsMin) && aligned && !sectors &&
-      (rp.L == 1 ? rp.R <= 32   // one lane: every slot coefficient is 0
-                 : rp.L == 2 && rp.V == 1 && rp.cl[0] == 1 && rp.grp_lanes >= 2 && rp.R <= kThreadRowsMax))
-    return ROWS_THREAD;
-  return rp.L > 1 || rp.R < 5 ? ROWS_TEAM : ROWS_NONE;
-}
-
 // launch of a rows kernel; its grid is sized on the nest's first run of that kind
 template <class Op, int V, bool DOT>
 hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const typename Op::In* A,
@@ -86,19 +67,6 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
   }
   const cudaError_t e = cudaPeekAtLastError();
   return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_rows_kernel launch");
-}
-
-// Does an item of this block-team plan lie in consecutive elements that
-// rect_flat_kernel can fold?  It also takes plain reductions of long rows from the
-// cp.async pipeline (2^26 elements, f32 / compensated / int64: rows of 4096 44, 54 and
-// 47 us there and 38, 44 and 39 here, 6400 51, 62, 59 and 39, 44, 39, 8192 43, 45, 44
-// and 40, 38, 37); the pipeline stays for dot products (compensated, 7168: 47 there,
-// 53 here) and 64-bit comparisons (5344: 50 and 52), for rows that a round of it
-// holds several of, and for other levels.
-inline bool flat_plan(const RectPlan& rp, bool leave) {
-  return rp.team == TEAM_BLOCK && rp.C == 1 && rp.W <= kFlatThreads / 32 && rp.nv == 1 && rp.vstride[0] == 1 &&
-         (!rp.pipe || (leave && rp.R >= 4096)) && rp.R >= 1 &&
-         (rp.G > 1 ? rp.split && rp.tile < (int64_t(1) << 30) : rp.R < (int64_t(1) << 30));
 }
 
 // the second pass over grid parts
@@ -157,10 +125,9 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
     return e == cudaSuccess ? HP_OK : cuda_fail(e, "rect_map_kernel launch");
   }
   if constexpr (Body::kPipeable) {
-    const RowsKind kind = rows_kind<Op, Body::kDot>(rp, body.A);
+    const RowsKind kind = rows_kind(np, (reinterpret_cast<uintptr_t>(body.A) & 15u) == 0);
     if (kind != ROWS_NONE) return launch_rows<Op, V, Body::kDot>(rp, kind, cfg, body.A, body.wptr(), a);
-    constexpr bool kCompare64 = std::is_same_v<Op, OpI64Max> || std::is_same_v<Op, OpI64Min>;
-    if (flat_plan(rp, !Body::kDot && !kCompare64)) return launch_flat<Op, V, Body::kDot>(rp, cfg, body.A, body.wptr(), a);
+    if (flat_plan(np)) return launch_flat<Op, V, Body::kDot>(rp, cfg, body.A, body.wptr(), a);
   }
   const bool block = rp.team == TEAM_BLOCK;
   constexpr bool kPipeable = Body::kPipeable && V == 4;
@@ -267,9 +234,7 @@ hp_status launch_team(const NestPlan& np, RectPlan rp, LaunchCfg& cfg, const Bod
     e = cudaPeekAtLastError();
     if (e != cudaSuccess) return cuda_fail(e, "rect_lanes_kernel launch");
   }
-  if (rp.G > 1) return launch_combine<Op>(rp, cfg.sms, a);
-  (void)np;
-  return HP_OK;
+  return rp.G > 1 ? launch_combine<Op>(rp, cfg.sms, a) : HP_OK;
 }
 
 template <class Op, class Body>
