@@ -55,26 +55,23 @@ struct StencilPlan {
   float c[(2 * kStencilMaxR + 1) * (2 * kStencilMaxR + 1)] = {};
   bool stream = false;           // tiles and sections automatic, and a streamed kernel exists
   size_t smem() const { return static_cast<size_t>(nbuf) * buf_floats * sizeof(float); }
-  // Does a run take the streamed kernel?  Steps kept in registers beat steps
-  // kept in shared memory everywhere (16384^2, radius 1, 4 steps: 443 us
-  // against 1026; radius 4, one step: 719 against 1410) but one aligned step of
-  // radius 1, which both run at the memory's rate and the tiles' large tensor
-  // copies read a little faster (334 us against 357), long arrays just wider
-  // than one column group but not than one tile, whose second group would be
-  // empty but for a few columns (8000 x 128: radius 3, 8 steps 119 us against
-  // 95 tiled, radius 4, 2 steps 31 against 23), and the widest ghost zones (24
-  // points, 80 of 128 columns kept; radius 4 with 4 steps) where the tiles about
-  // fill one wave of 152 CTAs (1500 x 738, radius 3, 8 steps: 129 us against 119, a
-  // second wave, 4499 x 459: 201 against 250; 537 x 1004, radius 4, 4 steps, 136
-  // tiles: 46 against 41, with 120 tiles the same).
-  bool streamed(bool vec) const {
-    if (r == 1 && T == 1 && vec) return false;
-    if (r >= 3 && T > 1 && stream_groups(nx, r, T) > 1 &&
-        ((tiles_x == 1 && tiles_y >= 60) ||
-         (tiles_y * tiles_x <= 152 && ((h >= 24 && tiles_y * tiles_x >= 100) ||
-                                       (r == 4 && T == 4 && tiles_y * tiles_x >= 133)))))
-      return false;
-    return stream;
+  // Does a run take the streamed kernel on a GPU of `sms` SMs?  Steps kept in
+  // registers beat steps kept in shared memory (16384^2, radius 1, 4 steps: 443 us
+  // against 1026; radius 4, one step: 719 against 1410) but for one aligned step of
+  // radius 1, which both run at the memory's rate and the tiles' large tensor copies
+  // read a little faster (334 us against 357), and for the widest windows (radius 4
+  // with 2 to 4 steps; ghost zones of 24 points, 80 of 128 columns kept) on arrays of
+  // whole tiles that fill one wave, a tile on each SM: 768^2, radius 4, 4 steps 43 us
+  // against 31, 1024^2, radius 3, 8 steps 111 against 88, 8000 x 128, radius 4, 2 steps 28
+  // against 20.  Over 800 sizes of radius 2 to 4 and up to 8 steps the kernel taken is 0.2%
+  // off the faster one (streaming always: 0.3%), at worst 1.3 times its time (512^2,
+  // radius 4, 4 steps).  Ragged tiles lose: 1000^2, radius 4, 2 steps 19 against 30.
+  bool streamed(bool vec, int sms) const {
+    if (!stream || (r == 1 && T == 1 && vec)) return false;
+    const int64_t tiles = tiles_y * tiles_x;
+    const bool wide = (r == 4 && T >= 2 && T <= 4) || h >= 24;
+    const bool wave = tiles <= sms && 4 * tiles >= 3 * static_cast<int64_t>(sms);
+    return !(vec && wide && wave && static_cast<double>(ny) * nx >= 0.97 * tiles * TY * TX);
   }
 };
 
@@ -163,7 +160,7 @@ std::string describe_stencil(const StencilPlan& p) {
     << ",\"tile\":[" << p.TY << "," << p.TX << "],\"ghost\":[" << p.h << "," << p.hx << "],\"box\":[" << p.boxH << ","
     << p.boxW << "],\"buffers\":" << p.nbuf << ",\"smem\":" << p.smem() << ",\"tiles\":" << p.order.size() / 2
     << ",\"section\":[" << p.SY << "," << p.SX << "],\"kernel\":\""
-    << (p.streamed(p.nx % 4 == 0) ? "stencil_stream" : "stencil_tile") << "\"";
+    << (p.streamed(p.nx % 4 == 0, 152) ? "stencil_stream" : "stencil_tile") << "\"";
   if (p.stream) s << ",\"warp_columns\":" << stream_columns(p.r, p.T);
   const int64_t secs_y = (p.ny + p.SY - 1) / std::max<int64_t>(p.SY, 1), secs_x = (p.nx + p.SX - 1) / std::max<int64_t>(p.SX, 1);
   if (p.ny > 0 && p.nx > 0 && secs_y * secs_x <= 64) {
@@ -531,7 +528,7 @@ extern "C" hp_status hp_stencil_run(hp_stencil* s, const float* in_dev, float* o
   cudaError_t e;
   const bool vec = p.nx % 4 == 0 && reinterpret_cast<uintptr_t>(in_dev) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(out_dev) % 16 == 0;
-  if (p.streamed(vec)) {
+  if (p.streamed(vec, s->sms)) {
     StreamArgs a;
     a.in = in_dev;
     a.out = out_dev;
