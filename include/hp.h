@@ -126,8 +126,9 @@ typedef enum hp_red_op {
  * quiet NaN 0x7fc00000 when there is none (the final value of a forward fill).
  * Exact (error bound 0).  Inputs 32-byte aligned with R (and grid parts) a
  * whole number of 256-bit loads use them; 16-byte aligned, 128-bit loads;
- * other rows are read as aligned 128-bit loads shifted in registers, for every
- * ordered operator, and short rows share a warp (the same pieces and tree).
+ * other maps and values with scalar loads or as aligned 128-bit loads shifted in
+ * registers, other matrices with scalar loads.  Many short rows share a warp (the
+ * same pieces and tree).
  */
 
 /*

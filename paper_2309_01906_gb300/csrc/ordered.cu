@@ -542,9 +542,8 @@ __global__ void __launch_bounds__(kOrdThreads) ordered_warp_kernel(OrdArgs g) {
 }
 
 // Rows of at most 16 pieces: L lanes per output (a power of two, one round of L
-// pieces holds the row), 32 / L outputs per warp.  The tree over L lanes is the
-// whole warp's without the levels that would only join identities.  4.8 M rows of
-// 7 maps: 918 us with a warp each, 51 here.
+// pieces holds the row), 32 / L outputs per warp, with the whole warp's tree.  4.8 M
+// rows of 7 maps: 918 us with a warp each, 51 here.
 template <class Op, int V>
 __global__ void __launch_bounds__(kOrdThreads) ordered_short_kernel(OrdArgs g, int L) {
   constexpr int64_t P = Op::template piece<V>();
@@ -556,7 +555,12 @@ __global__ void __launch_bounds__(kOrdThreads) ordered_short_kernel(OrdArgs g, i
     const int64_t s = std::min<int64_t>(lt * P, g.R), e = o < g.O ? std::min<int64_t>(s + P, g.R) : s;
     typename Op::S v = Op::template fold<V>(g, o * g.R, s, e, Op::ident());
     for (int m = 1; m < L; m <<= 1) v = Op::combine(v, Op::shfl(v, m));
-    v = Op::combine(Op::ident(), v);   // as the whole warp's round joins its running state
+    // the whole warp's other levels join identities on the right, and its round the
+    // running state on the left: they turn -0 into +0 and an infinite matrix entry into NaN
+    // (a third level changes nothing any more)
+    v = Op::combine(v, Op::ident());
+    if (L < 16) v = Op::combine(v, Op::ident());
+    v = Op::combine(Op::ident(), v);
     if (lt == 0 && o < g.O) Op::put(g.out, o, v);
   }
 }
