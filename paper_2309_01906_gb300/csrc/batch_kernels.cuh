@@ -545,6 +545,34 @@ __device__ __forceinline__ void ring_release(const RingView& r, int64_t lim, int
     if ((threadIdx.x & 31) == 0) mbar_arrive(r.empty + 8u * static_cast<uint32_t>(rel & (kStages - 1)));
 }
 
+// Reduce the partials of B items (part[r] = item r) over the L lanes of a
+// team in one go: recursive halving, each step handing half of the items to
+// the xor partner and combining the lower lane's partial first.  Every item
+// gets exactly the tree that lanes_allreduce builds at the team's lane 0, at
+// about one combine per item instead of log2(L).  On return part[0] of lane
+// lt holds item lt / (L / B) (B a power of two, B <= L).
+template <class Op, int B>
+__device__ __forceinline__ void lanes_reduce_many(typename Op::Acc (&part)[B], int L, int lt) {
+  using Acc = typename Op::Acc;
+  int m = L >> 1;
+#pragma unroll
+  for (int cnt = B; cnt > 1; cnt >>= 1, m >>= 1) {
+    const bool up = (lt & m) != 0;
+#pragma unroll
+    for (int i = 0; i < cnt / 2; ++i) {
+      const Acc send = up ? part[i] : part[i + cnt / 2];
+      const Acc keep = up ? part[i + cnt / 2] : part[i];
+      const Acc recv = Op::shfl_xor(send, m, L);
+      part[i] = up ? Op::combine(recv, keep) : Op::combine(keep, recv);
+    }
+  }
+  for (; m >= 1; m >>= 1) {
+    const Acc o = Op::shfl_xor(part[0], m, L);
+    part[0] = (lt & m) ? Op::combine(o, part[0]) : Op::combine(part[0], o);
+  }
+}
+constexpr int kReduceBatch = 4;   // items reduced together
+
 // block team, streamed.  Items go in chunks of up to kMaxM: each item is
 // folded in phases of whole steps (about two stages; a short remainder joins
 // the last phase), its warp partials are parked in shared memory, and after

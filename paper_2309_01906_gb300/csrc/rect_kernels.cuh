@@ -545,45 +545,16 @@ __global__ void __launch_bounds__(1024) rect_lanes_kernel(RectPlan p, Body body,
   }
 }
 
-// Reduce the partials of B items (part[r] = item r) over the L lanes of a
-// team in one go: recursive halving, each step handing half of the items to
-// the xor partner and combining the lower lane's partial first.  Every item
-// gets exactly the tree that lanes_allreduce builds at the team's lane 0, at
-// about one combine per item instead of log2(L).  On return part[0] of lane
-// lt holds item lt / (L / B) (B a power of two, B <= L).
-template <class Op, int B>
-__device__ __forceinline__ void lanes_reduce_many(typename Op::Acc (&part)[B], int L, int lt) {
-  using Acc = typename Op::Acc;
-  int m = L >> 1;
-#pragma unroll
-  for (int cnt = B; cnt > 1; cnt >>= 1, m >>= 1) {
-    const bool up = (lt & m) != 0;
-#pragma unroll
-    for (int i = 0; i < cnt / 2; ++i) {
-      const Acc send = up ? part[i] : part[i + cnt / 2];
-      const Acc keep = up ? part[i + cnt / 2] : part[i];
-      const Acc recv = Op::shfl_xor(send, m, L);
-      part[i] = up ? Op::combine(recv, keep) : Op::combine(keep, recv);
-    }
-  }
-  for (; m >= 1; m >>= 1) {
-    const Acc o = Op::shfl_xor(part[0], m, L);
-    part[0] = (lt & m) ? Op::combine(o, part[0]) : Op::combine(part[0], o);
-  }
-}
-constexpr int kReduceBatch = 4;   // items reduced together
-
-
 // ---------------------------------------------------------------- team = L lanes, whole rows
 // The plans that rect_lanes_kernel runs most, without its generality: one
 // reduced virtual level of stride 1 and no grid parts, so an output is a row of
-// R consecutive elements.  Every team folds U rows at once (row u of a warp's
-// set u) with U * NX row loads in flight; FP32 sums of one slot advance two rows
-// per packed FP32x2 instruction.  Each row sees the fold order and the reduction
-// tree of rect_lanes_kernel, so the bits are the same.  Bound by HBM for plain
-// sums (2^26 elements: rows of 64 and 1024, 51 and 47 us in the general kernel,
-// 41 here, 6.7 TB/s), by the compensated arithmetic's issue rate otherwise (dot
-// products of odd rows of 1021: 136 us, 72 here).
+// R consecutive elements.  A team folds one row (U = 1) with 4 positions loaded
+// ahead; a thread that is a team of its own folds U = 4 rows of at most 4 elements,
+// FP32 sums of one slot two rows per packed FP32x2 instruction.  Each row sees the
+// fold order and the reduction tree of rect_lanes_kernel, so the bits are the
+// same.  Bound by HBM for plain sums (2^26 elements: rows of 64 and 1024, 51 and 47 us
+// in the general kernel, 41 here, 6.7 TB/s), by the compensated arithmetic's issue
+// rate otherwise (dot products of odd rows of 1021: 136 us, 72 here).
 struct RowsArgs {
   int64_t O;
   int32_t R, P, L;             // elements per row, slots (elements per step), lanes per team
@@ -669,7 +640,7 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
   using Acc = typename Op::Acc;
   using In = typename Op::In;
   constexpr int NX = U == 1 ? 4 : 2;            // positions loaded before the first fold
-  const int L = g.L, R = g.R, P = g.P;
+  const int L = U > 1 ? 1 : g.L, R = g.R, P = g.P;
   const int lane = threadIdx.x & 31, lt = lane & (L - 1), set = 32 / L;
   const int s0 = (lt / g.grp_lanes) * g.cg + (lt % g.grp_lanes) * g.cl;
   const int64_t per = static_cast<int64_t>(set) * U;
@@ -714,17 +685,12 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
       // 511: 52 us, 72 so; f32 dot of 1200 x 3001: 10 us, 17 so)
       if constexpr (U == 1 && !DOT && !std::is_same_v<Acc, f2>) {
         if (x < R) {
-          Vals<Op, V> v[NX - 1][U];
-          In b[NX - 1][V];
+          Vals<Op, V> v[NX - 1][1];
 #pragma unroll
-          for (int q = 0; q < NX - 1; ++q) {
-            const int y = x + q * P < R ? x + q * P : x;
-            if constexpr (DOT) load_bcast<In, V>(w + y, b[q]);
-            load_row<In, V>(a + y, v[q][0].a);
-          }
+          for (int q = 0; q < NX - 1; ++q) load_row<In, V>(a + (x + q * P < R ? x + q * P : x), v[q][0].a);
 #pragma unroll
           for (int q = 0; q < NX - 1; ++q)
-            if (x + q * P < R) fold_rows<Op, V, DOT, U>(acc, v[q], b[q]);
+            if (x + q * P < R) fold_vals_load<Op, V>(acc[0], v[q][0].a);
           x = R;
         }
       }
@@ -742,25 +708,14 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
     Acc part[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) part[u] = fold_vec<Op, V>(acc[u]);
-    if (U > 1 && L >= U) {
-      lanes_reduce_many<Op, U>(part, L, lt);
-      const int64_t o = row + static_cast<int64_t>(lt / (L / U)) * set;
-      if ((lt & (L / U - 1)) == 0 && o < g.O) {
-        out[o] = Op::finish(part[0]);
-        if constexpr (std::is_same_v<Acc, f2>) {
-          if (comp) comp[o] = Op::residual(part[0]);
-        }
-      }
-    } else {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const Acc r = lanes_allreduce<Op>(part[u], L);
-        const int64_t o = row + static_cast<int64_t>(u) * set;
-        if (lt == 0 && o < g.O) {
-          out[o] = Op::finish(r);
-          if constexpr (std::is_same_v<Acc, f2>) {
-            if (comp) comp[o] = Op::residual(r);
-          }
+    for (int u = 0; u < U; ++u) {
+      const Acc r = lanes_allreduce<Op>(part[u], L);
+      const int64_t o = row + static_cast<int64_t>(u) * set;
+      if (lt == 0 && o < g.O) {
+        out[o] = Op::finish(r);
+        if constexpr (std::is_same_v<Acc, f2>) {
+          if (comp) comp[o] = Op::residual(r);
         }
       }
     }

@@ -67,7 +67,7 @@ struct StencilPlan {
   // off the faster one (streaming always: 0.3%), at worst 1.3 times its time (512^2,
   // radius 4, 4 steps).  Ragged tiles lose: 1000^2, radius 4, 2 steps 19 against 30.
   bool streamed(bool vec, int sms) const {
-    if (!stream || (r == 1 && T == 1 && vec)) return false;
+    if (!stream || !stream_has(r, T, vec)) return false;
     const int64_t tiles = tiles_y * tiles_x;
     const bool wide = (r == 4 && T >= 2 && T <= 4) || h >= 24;
     const bool wave = tiles <= sms && 4 * tiles >= 3 * static_cast<int64_t>(sms);
@@ -483,7 +483,8 @@ hp_status stencil_ensure_device(hp_stencil* s) {
   if ((e = cudaMalloc(&s->err, sizeof(int32_t))) != cudaSuccess) return fail(HP_ENOMEM, "cudaMalloc (error word)");
   if ((e = init.zero(s->err, sizeof(int32_t))) != cudaSuccess) return stencil_cuda_fail(e, "clear error word");
   const StencilPlan& p = s->plan;
-  for (int vec = 0; p.stream && vec < 2; ++vec) {
+  for (int vec = 0; vec < 2; ++vec) {
+    if (!p.stream || !stream_has(p.r, p.T, vec != 0)) continue;
     const int ctas = stream_occupancy(p.r, p.T, vec != 0, &e);
     if (e != cudaSuccess) return stencil_cuda_fail(e, "occupancy query");
     s->strip[vec] = stream_strip_rows(p.ny, p.nx, p.r, p.T, std::max(ctas, 1), s->sms);

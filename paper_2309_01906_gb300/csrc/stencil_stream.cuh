@@ -254,7 +254,9 @@ constexpr auto stream_kernel() {
 template <int R, bool VEC, int T = 1>
 auto stream_pick(int t) -> void (*)(const StreamArgs) {
   if constexpr (stream_has(R, T)) {
-    if (t == T) return stream_kernel<R, T, VEC>();
+    if constexpr (stream_has(R, T, VEC)) {
+      if (t == T) return stream_kernel<R, T, VEC>();
+    }
     return stream_pick<R, VEC, T + 1>(t);
   }
   return nullptr;

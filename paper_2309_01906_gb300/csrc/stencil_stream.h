@@ -23,6 +23,9 @@ struct StreamArgs {
 // tiled kernel's rate).
 constexpr bool stream_has(int R, int T) { return R >= 1 && R <= 3 ? T >= 1 && T <= 8 : R == 4 && T >= 1 && T <= 5; }
 
+// One aligned step of radius 1 stays tiled.
+constexpr bool stream_has(int R, int T, bool vec) { return stream_has(R, T) && !(vec && R == 1 && T == 1); }
+
 // CTAs of the kernel that fit on an SM (0 if none; CUDA error in *e)
 int stream_occupancy(int R, int T, bool vec, cudaError_t* e);
 
