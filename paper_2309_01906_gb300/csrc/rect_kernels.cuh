@@ -559,6 +559,13 @@ struct RowsArgs {
   int64_t O;
   int32_t R, P, L;             // elements per row, slots (elements per step), lanes per team
   int32_t grp_lanes, cg, cl;   // slot of lane lt: (lt / grp_lanes) * cg + (lt % grp_lanes) * cl
+  // One row at a time: teams past the last row fold it once more and store nothing, so
+  // that a last warp that is not full keeps its loads in flight (500 rows of 101 f32:
+  // 5.9 us a position at a time, 3.2 us in rect_lanes_kernel).  An argument, not a
+  // constant: where the compiler knew the single positions' loop to be unreachable,
+  // the others' schedule took 3 to 9% longer (300,000 rows of 500 f32: 90 us, 98 so).
+  // Compensated dot products have no registers for it (146 us, 164 so).
+  int32_t again;
 };
 constexpr int kRowsThreads = 256;
 
@@ -640,6 +647,7 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
   using Acc = typename Op::Acc;
   using In = typename Op::In;
   constexpr int NX = U == 1 ? 4 : 2;            // positions loaded before the first fold
+  constexpr bool kAgain = U == 1 && !(DOT && std::is_same_v<Acc, f2>);
   const int L = U > 1 ? 1 : g.L, R = g.R, P = g.P;
   const int lane = threadIdx.x & 31, lt = lane & (L - 1), set = 32 / L;
   const int s0 = (lt / g.grp_lanes) * g.cg + (lt % g.grp_lanes) * g.cl;
@@ -648,17 +656,19 @@ __global__ void __launch_bounds__(kRowsThreads, (rows_blocks<Op, V, DOT, U>()))
   for (int64_t base = (static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per; base < g.O;
        base += stride) {
     const int64_t row = base + lane / L;
-    // one row at a time, teams past the last row fold it once more and store nothing:
-    // the whole warp keeps its loads in flight (500 rows of 101 f32, the last warp half
-    // full: 5.9 us a position at a time, 3.2 us in rect_lanes_kernel)
-    const In* a = A + (U == 1 && row >= g.O ? g.O - 1 : row) * R;
+    const bool full = base + per <= g.O;        // the same in every lane
+    int64_t from = row;
+    if constexpr (kAgain) {
+      if (!full && g.again && row >= g.O) from = g.O - 1;
+    }
+    const In* a = A + from * R;
     const int dist = set * R;                   // elements between a team's rows
     Acc acc[U][V];
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int i = 0; i < V; ++i) acc[u][i] = Op::ident();
-    const bool whole = U == 1 || base + per <= g.O;   // the same in every lane
+    const bool whole = full || (kAgain && g.again);
     int rows = U;                               // this lane's rows
     if (!whole) {
       rows = 0;

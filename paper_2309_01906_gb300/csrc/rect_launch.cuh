@@ -61,7 +61,7 @@ hp_status launch_rows(const RectPlan& rp, RowsKind kind, LaunchCfg& cfg, const t
   if (kind == ROWS_THREAD) {
     kt<<<grid, kRowsThreads, dyn, a.stream>>>(rp.O, static_cast<int>(rp.R), rp.L, K, A, w, out, a.comp);
   } else {
-    const RowsArgs g{rp.O, static_cast<int32_t>(rp.R), rp.vP[0], rp.L, rp.grp_lanes, rp.cg[0], rp.cl[0]};
+    const RowsArgs g{rp.O, static_cast<int32_t>(rp.R), rp.vP[0], rp.L, rp.grp_lanes, rp.cg[0], rp.cl[0], U == 1 ? 1 : 0};
     if (U == 1) k1<<<grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
     else k4<<<grid, kRowsThreads, 0, a.stream>>>(g, A, w, out, a.comp);
   }
