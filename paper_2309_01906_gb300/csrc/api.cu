@@ -4,6 +4,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -18,6 +19,17 @@ const std::string& last_error_string();
 uint64_t next_plan_id() {
   static std::atomic<uint64_t> counter{0};
   return ++counter;
+}
+
+cudaStream_t init_stream() {
+  constexpr int kDevices = 64;
+  static std::mutex mu;
+  static cudaStream_t streams[kDevices] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!streams[dev] && cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking) != cudaSuccess) streams[dev] = nullptr;
+  return streams[dev];
 }
 
 hp_status ensure_device(hp_nest* n, const cudaStream_t* run) {
