@@ -56,10 +56,10 @@ struct StencilPlan {
   bool stream = false;           // tiles and sections automatic, and a streamed kernel exists
   size_t smem() const { return static_cast<size_t>(nbuf) * buf_floats * sizeof(float); }
   // Does a run take the streamed kernel on a GPU of `sms` SMs?  Steps kept in
-  // registers beat steps kept in shared memory (16384^2, radius 1, 4 steps: 443 us
-  // against 1026; radius 4, one step: 719 against 1410) but for one aligned step of
+  // registers beat steps kept in shared memory (16384^2, radius 1, 4 steps: 439 us
+  // against 1024; radius 4, one step: 720 against 1261) but for one aligned step of
   // radius 1, which both run at the memory's rate and the tiles' large tensor copies
-  // read a little faster (334 us against 357), and for the widest windows (radius 4
+  // read a little faster (326 us, with 2 steps streamed 357), and for the widest windows (radius 4
   // with 2 to 4 steps; ghost zones of 24 points, 80 of 128 columns kept) on arrays of
   // whole tiles that fill one wave, a tile on each SM: 768^2, radius 4, 4 steps 43 us
   // against 31, 1024^2, radius 3, 8 steps 111 against 88, 8000 x 128, radius 4, 2 steps 28

@@ -18,11 +18,12 @@
 // Rows arrive through a ring of D stages per warp filled by cp.async (absent
 // rows and columns are zero-filled by the copy), D - 2 rows ahead.
 //
-// What bounds it: HBM up to 36 FMAs per point (16384^2, radius 1: 1 to 3 steps
-// 355 to 370 us, 5.8-6.1 TB/s; radius 2, one step 357 us against 680 tiled),
-// FMA issue beyond (radius 1: 4 steps 443 us = 44 TFLOP/s against 1026 us tiled,
-// 8 steps 989; radius 4, one step: 719 us = 60 TFLOP/s against 1410 tiled).  The
-// tiled kernel read each window row from shared memory, 2R + 1 loads a point.
+// What bounds it: HBM up to 36 FMAs per point (16384^2, radius 1: 2 and 3 steps
+// 357 us, 6.0 TB/s; radius 2, one step 351 us against 536 tiled), instruction issue
+// beyond (radius 1: 4 steps 439 us = 44 TFLOP/s against 1024 us tiled, 8 steps 916
+// against 2408; radius 4, one step: 720 us = 60 TFLOP/s against 1261 tiled; 4 steps of
+// radius 1 use 0.80 of the issue slots and keep the FMA pipe active 0.61 of the
+// time).  The tiled kernel reads each window row from shared memory, 2R + 1 loads a point.
 // Packed FP32x2 FMAs over two strips per warp measured no faster than scalar
 // ones (4 steps 483 us) and were left out.  128 columns per warp: a narrower
 // group would spend more of its lanes on ghost columns (4 steps of radius 1: 8
@@ -236,8 +237,8 @@ __global__ void __launch_bounds__(32 * kStreamWarps, MINB)
 
 // Registers grow with the partial sums (8 R T) and the window; the CTAs per SM
 // that each kernel is compiled for were swept one up and one down at 16384^2
-// (e.g. radius 1: 4 steps 6 CTAs 443 us, 7 CTAs 450, 8 CTAs 487; 8 steps 3 CTAs 989 us, 4
-// CTAs 1011; radius 2: 4 steps 3 CTAs 1191 us, 4 CTAs 1265).
+// with strips of one length (e.g. radius 1: 4 steps 6 CTAs 443 us, 7 CTAs 450, 8 CTAs
+// 487; 8 steps 3 CTAs 989 us, 4 CTAs 1011; radius 2: 4 steps 3 CTAs 1191 us, 4 CTAs 1265).
 constexpr int stream_blocks(int R, int T) {
   const int q = 8 * R * T + 4 * R;
   return T == 1 ? (R <= 2 ? 8 : R == 3 ? 6 : 7) : q <= 20 ? 8 : q <= 36 ? 6 : q <= 44 ? 5 : q <= 60 ? 4 : q <= 104 ? 3 : 2;
