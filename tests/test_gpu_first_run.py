@@ -74,3 +74,28 @@ def test_first_run_on_a_stream_of_its_own(kind):
     assert n.check(side.cuda_stream) == 0
     torch.cuda.synchronize()
     n.close()
+
+
+@pytest.mark.parametrize("kind", ["csr", "csr_hist", "narrow", "last", "rect"])
+def test_first_run_inside_a_capture(kind):
+    """A relaxed capture may hold a nest's first run: what it finds is ready at once, not only after a replay."""
+    import torch
+    n, ins, out, want = _csr(kind == "csr_hist") if kind.startswith("csr") else _split(kind)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin(capture_error_mode="relaxed")
+        n.run([t.data_ptr() for t in ins], out.data_ptr(), side.cuda_stream)
+        graph.capture_end()
+        for replay in (False, True, True, False, True):
+            out.fill_(7)
+            if replay:
+                graph.replay()
+            else:
+                n.run([t.data_ptr() for t in ins], out.data_ptr(), side.cuda_stream)
+            side.synchronize()
+            assert torch.equal(out.cpu(), want)
+    assert n.check(side.cuda_stream) == 0
+    del graph
+    n.close()
