@@ -56,12 +56,15 @@ constexpr int64_t kCsrChunk = HP_CSR_CHUNK;
 static_assert(kCsrLimit3 >= kCsrChunk, "split rows must be longer than one chunk (bounds the chunk slots)");
 constexpr int kCsrThreads = 256;                          // every kernel's CTA
 // rows of one unit of work, by class: a chunk, a row, up to kCsrWarpRows rows per
-// warp, 8 rows per 8-lane team, 8 rows per thread
-constexpr int kCsrUnit0 = 8 * kCsrThreads, kCsrUnit1 = kCsrThreads, kCsrWarps = kCsrThreads / 32;
-// fewer where a CTA would not get 8 units (rows of 2000, 4 rows per warp and now: 5000
-// rows, 157 units for 760 CTAs, 119 and 56 us; 50,000, whose 1562 units leave a last
-// wave nearly empty, 446 and 379)
-constexpr int kCsrWarpRows = 4;
+// warp, up to kCsrTeamRows rows per 8-lane team, 8 rows per thread
+constexpr int kCsrUnit0 = 8 * kCsrThreads, kCsrWarps = kCsrThreads / 32, kCsrTeams = kCsrThreads / 8;
+// fewer where the CTAs would not get a unit each (rows of 64: 300 rows 22 and 11 us in
+// a graph) or, when the nest's rows are long enough to hide a unit's claim, 8 each
+// (rows of 2000, 4 rows per warp and now: 5000 rows, 157 units for 760 CTAs, 119 and 56 us;
+// 50,000, whose 1562 units leave a last wave nearly empty, 446 and 379; rows of 100, 8 units
+// each: 57 and 61)
+constexpr int kCsrWarpRows = 4, kCsrTeamRows = 8;
+constexpr int64_t kCsrLongRows = 512;   // entries per row, on average
 // up to this many chunk slots the last CTA of the work kernel folds the long
 // rows' partials; beyond, a kernel of its own does (25,000 rows would take one
 // CTA about 200 us)
@@ -454,6 +457,7 @@ struct CsrLists {
   const int32_t* chunk_cnt;
   int64_t n_rows, max_chunks;
   int tail_combine;           // 1: the last CTA folds the long rows' partials
+  uint32_t units;             // of the warp class, per CTA, that its rows per warp leave
 };
 
 // All classes in one persistent kernel: units are taken from a counter, chunks
@@ -468,7 +472,7 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
   using Acc = typename Op::Acc;
   extern __shared__ int sh_hist[];
   __shared__ Acc wsh[2][kCsrThreads / 32];
-  __shared__ uint32_t s_unit, s_first[kCsrClasses], s_rows[3], s_per, s_end;   // s_per: class 2's rows per warp
+  __shared__ uint32_t s_unit, s_first[kCsrClasses], s_rows[3], s_per[3], s_end;   // s_per: rows per team and unit
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned long long* const claim = reinterpret_cast<unsigned long long*>(&l.counters[kCntUnit]);
@@ -485,11 +489,13 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
     s_first[4] = 0;
     s_first[3] = static_cast<uint32_t>(slots);
     s_first[2] = s_first[3] + static_cast<uint32_t>(min(l.counters[3], l.n_rows));
-    uint32_t per = kCsrWarpRows;
-    while (per > 1 && s_rows[2] < 8 * gridDim.x * (kCsrWarps * per)) per /= 2;
-    s_per = per;
-    s_first[1] = s_first[2] + (s_rows[2] + kCsrWarps * per - 1) / (kCsrWarps * per);
-    s_first[0] = s_first[1] + (s_rows[1] + kCsrUnit1 - 1) / kCsrUnit1;
+    for (int c = 2; c >= 1; --c) {
+      const uint32_t teams = c == 2 ? kCsrWarps : kCsrTeams;
+      uint32_t per = c == 2 ? kCsrWarpRows : kCsrTeamRows;
+      while (per > 1 && s_rows[c] < (c == 2 ? l.units : 1) * gridDim.x * (teams * per)) per /= 2;
+      s_per[c] = per;
+      s_first[c - 1] = s_first[c] + (s_rows[c] + teams * per - 1) / (teams * per);
+    }
     s_end = s_first[0] + (s_rows[0] + kCsrUnit0 - 1) / kCsrUnit0;
   }
   __syncthreads();
@@ -520,8 +526,8 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
         if (chunk) part[u] = r;
         else a.y[row] = Op::finish(r);
       }
-    } else if (u < s_first[1]) {   // s_per rows per warp; lane i reads the i-th one's place
-      const uint32_t per = s_per, k0 = ((u - s_first[2]) * kCsrWarps + warp) * per;
+    } else if (u < s_first[1]) {   // `per` rows per warp; lane i reads the i-th one's place
+      const uint32_t per = s_per[2], k0 = ((u - s_first[2]) * kCsrWarps + warp) * per;
       const int n = k0 >= s_rows[2] ? 0 : static_cast<int>(min(s_rows[2] - k0, per));
       int32_t id = 0;
       int64_t s = 0, e = 0;
@@ -538,16 +544,16 @@ __global__ void __launch_bounds__(kCsrThreads, HP_CSR_MIN_BLOCKS) csr_work_kerne
         const Acc r = team_reduce<Op>(fold4<Op>(acc), 32);
         if (lane == i) a.y[id] = Op::finish(r);
       }
-    } else if (u < s_first[0]) {   // 8 lanes per row, 32 rows per warp
-      const uint32_t k0 = (u - s_first[1]) * kCsrUnit1 + warp * 32;
+    } else if (u < s_first[0]) {   // 8 lanes per row, 4 `per` rows per warp
+      const uint32_t per = s_per[1], k0 = ((u - s_first[1]) * kCsrWarps + warp) * (4 * per);
       int32_t id = -1;
       int64_t s = 0, e = 0;
-      if (k0 + lane < s_rows[1]) {
+      if (lane < 4 * per && k0 + lane < s_rows[1]) {
         id = l.rows01[list_at(1, k0 + lane, l.n_rows)];
         s = a.off[id];
         e = a.off[id + 1];
       }
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < static_cast<int>(per); ++i) {
         const int src = 4 * i + (lane >> 3);
         const int32_t row = __shfl_sync(0xffffffffu, id, src);
         const int64_t rs = __shfl_sync(0xffffffffu, s, src), re = __shfl_sync(0xffffffffu, e, src);
@@ -662,7 +668,7 @@ struct CsrRun {
     const CsrState& cs = *n->cs;
     const bool tail = cs.max_chunks <= kCsrTailChunks;
     const CsrLists l{cs.counters, cs.rows01, cs.rows23, cs.chunk_row, cs.chunk_idx, cs.chunk_cnt,
-                     n->csr.n_rows, cs.max_chunks, tail ? 1 : 0};
+                     n->csr.n_rows, cs.max_chunks, tail ? 1 : 0, n->csr.nnz >= kCsrLongRows * n->csr.n_rows ? 8u : 1u};
     typename Op::Acc* part = static_cast<typename Op::Acc*>(cs.part);
     const cudaError_t w = launch_dependent(csr_work_kernel<Op, HIST>, cs.grid, kCsrThreads, dyn(), st, a, l, part);
     if (w != cudaSuccess) return cuda_fail(w, "CSR work kernel launch");

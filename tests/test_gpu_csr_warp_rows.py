@@ -1,6 +1,6 @@
-"""GPU test of CSR rows that take a warp each, around the row counts at which a unit
-of work holds 1, 2 and 4 of them per warp (760 CTAs with 8 units each).  Small
-integers, so FP32 sums are exact."""
+"""GPU test of CSR rows that take a warp or 8 lanes each, around the row counts at
+which a unit of work holds 1, 2, 4 (and 8) of them per team (760 CTAs with a unit
+each, 8 for long rows).  Small integers, so FP32 sums are exact."""
 import numpy as np
 import pytest
 
@@ -9,12 +9,14 @@ from paper_2309_01906_gb300 import binding as hb
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("rows", [9, 97279, 97281, 97296, 194559, 194561, 194592])
+@pytest.mark.parametrize("rows,ln", [(9, 67), (12159, 600), (12161, 67), (24319, 67), (24321, 300), (97279, 520), (97281, 520),
+                                     (97296, 67), (194561, 67), (1, 20), (33, 64), (48639, 64), (48641, 64), (97279, 50),
+                                     (97281, 50), (194559, 20), (194561, 20), (389121, 5)])
 @pytest.mark.parametrize("fuse", [0, 1])
-def test_rows_per_warp(rows, fuse):
+def test_rows_per_team(rows, ln, fuse):
     import torch
     g = torch.Generator("cuda").manual_seed(rows)
-    ln, cols = 67, 2000
+    cols = 2000
     off = torch.arange(rows + 1, device="cuda") * ln
     col = torch.randint(0, cols, (rows * ln,), dtype=torch.int32, device="cuda", generator=g)
     val, x = (torch.randint(-2, 3, (k,), device="cuda", generator=g).float() for k in (rows * ln, cols))
